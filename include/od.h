@@ -142,8 +142,10 @@ typedef struct od_config {
                                     (and 256x8 for rows past 1024 cells) by
                                     the lanes its tiles use, the halo rows and
                                     the tile count, preferring 128x4 */
-    int32_t stages;              /* TMA ring slots, 3..8 (0 = 4): planes k-1,
-                                    k, k+1 resident, the rest in flight */
+    int32_t stages;              /* TMA ring slots, 3..8: planes k-1, k, k+1
+                                    resident, the rest in flight (0 = 4, with
+                                    the default arithmetic as many as the shared
+                                    memory holds, up to 6 in 3D and 8 in 2D) */
     int32_t arith;               /* where the update's operations run (the bits
                                     never change): 0 all on the FP64 pipe;
                                     1 division by 6 on the integer pipes;
@@ -159,6 +161,11 @@ typedef struct od_config {
                                     largest value (see od_write); 13: one FP64
                                     add, four window adds; 14 / 15: 13 on every
                                     other / every fourth cell, 12 on the rest.
+                                    Mode 12 keeps the field itself as words of
+                                    such a window where it can (from od_create
+                                    or od_write on; until a face is imported or
+                                    a field reaches 2^757) and then needs no
+                                    FP64 add.
                                     2D: 12 one FP64 add and two window adds,
                                     13 none and three, 14 the two mixed, 15
                                     two FP64 adds and one window add.  -1 =
@@ -486,7 +493,7 @@ typedef struct od_server_config {
                                     cells_per_thread both 0: the planner picks
                                     each job's shape (as od_config; batched mode
                                     runs one launch per shape in use); stages
-                                    0 = 4 */
+                                    0 = 4 (per-job launches: as od_config) */
     int32_t arith;               /* as od_config.arith (-1 = 12) */
     void *pool;                  /* caller device memory of hbm_budget_bytes, 256-byte
                                     aligned, or NULL: the server allocates it once */

@@ -74,8 +74,11 @@ KArgs base_args_impl(const od_ctx *c) {
     a.epoch = c->d_epoch;
     a.dep_ptr = c->d_dep_ptr;
     a.dep_idx = c->d_dep_idx;
-    a.order = c->d_order;
+    // the sweep over words takes index order without a table
+    a.order = c->words && !(c->cfg.order & 2) ? nullptr : c->d_order;
     a.vmax = c->d_vmax;
+    a.fmt = c->d_fmt;
+    a.rec = c->d_rec;
     a.one = 1u;
     a.ntiles = (int32_t)c->plan.tiles.size();
     a.order_mode = c->cfg.order & 1;
@@ -94,7 +97,8 @@ od_status enqueue_fused(od_ctx *c, int32_t iters) {
         KArgs a = base_args_impl(c);
         a.tile_begin = 0;
         a.parity = (int32_t)(c->steps & 1);
-        OD_CUDA(od::launch_tiles(a, (int)p.tiles.size(), p.threads, p.cpt, p.amode, true, p.smem_bytes, c->stream));
+        OD_CUDA(od::launch_tiles(a, (int)p.tiles.size(), p.threads, p.cpt, c->kernel_mode(), true, p.smem_bytes,
+                                 c->resident, c->stream));
         c->steps++;
         c->launches++;
         c->api_calls++;
@@ -107,7 +111,7 @@ od_status enqueue_persistent(od_ctx *c, int32_t iters) {
     const od::Plan &p = c->plan;
     const int64_t nt = (int64_t)p.tiles.size();
     int bps = 0;
-    OD_CUDA(od::persistent_occupancy(p.threads, p.cpt, p.amode, p.smem_bytes, p.stencil, &bps));
+    OD_CUDA(od::persistent_occupancy(p.threads, p.cpt, c->kernel_mode(), p.smem_bytes, p.stencil, &bps));
     if (bps < 1) return fail(OD_EINVAL, "persistent kernel does not fit on an SM with this tiling");
     int grid = (int)std::min<int64_t>(nt, (int64_t)bps * c->num_sms);
     c->persistent_grid = grid;
@@ -121,7 +125,7 @@ od_status enqueue_persistent(od_ctx *c, int32_t iters) {
         KArgs a = base_args_impl(c);
         a.iters = n;
         a.t0 = (int32_t)(c->steps & 0x7fffffff);
-        OD_CUDA(od::launch_persistent(a, grid, p.threads, p.cpt, p.amode, p.smem_bytes, c->stream));
+        OD_CUDA(od::launch_persistent(a, grid, p.threads, p.cpt, c->kernel_mode(), p.smem_bytes, c->stream));
         c->steps += n;
         c->launches++;
         c->api_calls += 3;
@@ -147,7 +151,8 @@ cudaError_t per_chare_phase_a(od_ctx *c, int ci, int64_t t, cudaStream_t st, int
     KArgs a = base_args_impl(c);
     a.tile_begin = h.tile_begin;
     a.parity = sp;
-    cudaError_t e = od::launch_tiles(a, h.tile_end - h.tile_begin, p.threads, p.cpt, p.amode, false, p.smem_bytes, st);
+    cudaError_t e = od::launch_tiles(a, h.tile_end - h.tile_begin, p.threads, p.cpt, c->kernel_mode(), false,
+                                    p.smem_bytes, c->resident, st);
     if (e == cudaSuccess) e = od::launch_pack(c->d_ch, ci, dp, h.foff[6], st);
     if (e != cudaSuccess) return e;
     (*kernels) += 2;
@@ -363,7 +368,8 @@ od_status capture_fused(od_ctx *c, int64_t t_first, int32_t iters, cudaGraphExec
         KArgs a = base_args_impl(c);
         a.tile_begin = 0;
         a.parity = (int32_t)((t_first + s) & 1);
-        e = od::launch_tiles(a, (int)p.tiles.size(), p.threads, p.cpt, p.amode, true, p.smem_bytes, c->stream);
+        e = od::launch_tiles(a, (int)p.tiles.size(), p.threads, p.cpt, c->kernel_mode(), true, p.smem_bytes,
+                                 c->resident, c->stream);
     }
     const cudaError_t e2 = cudaStreamEndCapture(c->stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -473,14 +479,19 @@ od_status ensure_stage(od_ctx *c) {
     return OD_OK;
 }
 
+// The captured step loops (they are captured again when next needed).
+void drop_graphs(od_ctx *c) {
+    for (cudaGraphExec_t *g : {&c->g2, &c->g1[0], &c->g1[1], &c->gf, &c->gf1[0], &c->gf1[1]}) {
+        if (*g) cudaGraphExecDestroy(*g);
+        *g = nullptr;
+    }
+    c->g2_kernels = c->g1_kernels[0] = c->g1_kernels[1] = 0;
+    c->g2_calls = c->g1_calls[0] = c->g1_calls[1] = 0;
+}
+
 void release(od_ctx *c) {
     if (!c) return;
-    if (c->g2) cudaGraphExecDestroy(c->g2);
-    for (auto &g : c->g1)
-        if (g) cudaGraphExecDestroy(g);
-    if (c->gf) cudaGraphExecDestroy(c->gf);
-    for (auto &g : c->gf1)
-        if (g) cudaGraphExecDestroy(g);
+    drop_graphs(c);
     for (auto e : c->ev) cudaEventDestroy(e);
     for (auto e : c->join) cudaEventDestroy(e);
     if (c->fork) cudaEventDestroy(c->fork);
@@ -549,9 +560,9 @@ std::string tune_key(const od_config *cfg, const od::Plan &p, int device) {
     mix(-1);
     for (auto v : p.ez) mix(v);
     char buf[256];
-    // "k2": the kernel generation (pulled 3D halos, anchored arithmetic); an
+    // "k3": the kernel generation (pulled 3D halos, fixed-point field words); an
     // entry timed on another generation's kernels is not reused
-    snprintf(buf, sizeof buf, "k2/%s/%d/path%d/st%d/%lldx%lldx%lld/%016llx", name.c_str(), sms, cfg->path,
+    snprintf(buf, sizeof buf, "k3/%s/%d/path%d/st%d/%lldx%lldx%lld/%016llx", name.c_str(), sms, cfg->path,
              p.stencil, (long long)p.nx, (long long)p.ny, (long long)p.nz, (unsigned long long)h);
     return buf;
 }
@@ -937,6 +948,8 @@ od_status create_context(od_ctx **out, const od_config *cfg_in, bool sync) {
     c->d_dep_idx = (int32_t *)(A + p.off_dep_idx);
     c->d_order = (int32_t *)(A + p.off_order);
     c->d_vmax = (uint64_t *)(A + p.off_queue + 8);  // the queue block holds 64 bytes
+    c->d_fmt = (FmtDev *)(A + p.off_queue + 16);
+    c->words = p.amode == od::kDefaultArith;
     c->h_ch.resize(p.ch.size());
     for (size_t i = 0; i < p.ch.size(); ++i) {
         const od::HostChare &h = p.ch[i];
@@ -965,7 +978,21 @@ od_status create_context(od_ctx **out, const od_config *cfg_in, bool sync) {
                                cudaMemcpyHostToDevice, c->stream));
     OD_TRY(cudaMemcpyAsync(c->d_order, p.order.data(), p.order.size() * sizeof(int32_t),
                            cudaMemcpyHostToDevice, c->stream));
+    if (c->words) {
+        c->d_rec = (TileRec *)(A + p.off_rec);
+        OD_TRY(od::launch_tile_recs(c->d_ch, c->d_tiles, (int64_t)p.tiles.size(), c->d_dep_ptr, c->d_dep_idx, c->d_rec,
+                                    p.stencil, c->stream));
+    }
     OD_TRY(od::prepare_tile_kernels(p.threads, p.cpt, p.amode, p.smem_bytes, p.stencil));
+    if (c->words) {
+        // a ring that leaves no room for those kernels' own shared memory runs plain doubles
+        const int km = c->kernel_mode();
+        int bps = 0;
+        if (od::prepare_tile_kernels(p.threads, p.cpt, km, p.smem_bytes, p.stencil) == cudaSuccess)
+            OD_TRY(od::tiles_occupancy(p.threads, p.cpt, km, p.smem_bytes, p.stencil, &bps));
+        c->resident = bps * c->num_sms;
+        c->words = bps > 0;
+    }
     // per-chare path resources
     int P = cfg->stream_pool > 0 ? cfg->stream_pool : 32;
     P = (int)std::min<int64_t>(P, (int64_t)p.ch.size());
@@ -978,13 +1005,17 @@ od_status create_context(od_ctx **out, const od_config *cfg_in, bool sync) {
     OD_TRY(cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming));
     c->ev.resize(2 * p.ch.size(), nullptr);
     for (auto &e : c->ev) OD_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    OD_TRY(od::launch_init(c->d_ch, (int)p.ch.size(), p.gnx, p.gny, p.gnz, p.gx0, p.gy0, p.gz0, cfg->seed,
-                           cfg->init_mode, p.stencil,
-                           c->stream));
     // every initial value lies in [0, 1): the largest possible one anchors
     // the exact arithmetic's window (od_write raises it for imported fields)
-    const uint64_t vmax0 = 0x3FEFFFFFFFFFFFFFull;
-    OD_TRY(cudaMemcpyAsync(c->d_vmax, &vmax0, sizeof vmax0, cudaMemcpyHostToDevice, c->stream));
+    // and, where the field is kept as words, their format
+    struct {
+        uint64_t vmax;
+        FmtDev fmt;
+    } head = {0x3FEFFFFFFFFFFFFFull, {0u, 0u}};
+    if (c->words) head.fmt.base = od::fx_anchor(head.vmax);
+    OD_TRY(cudaMemcpyAsync(c->d_vmax, &head, sizeof head, cudaMemcpyHostToDevice, c->stream));
+    OD_TRY(od::launch_init(c->d_ch, (int)p.ch.size(), p.gnx, p.gny, p.gnz, p.gx0, p.gy0, p.gz0, cfg->seed,
+                           cfg->init_mode, p.stencil, head.fmt.base, c->stream));
     if (sync) OD_TRY(cudaStreamSynchronize(c->stream));
     c->ghosts_current = true;
 #undef OD_TRY
@@ -1074,7 +1105,7 @@ od_status od_read_cells(od_ctx *c, const int64_t *cells, int64_t n, double *out)
         e = cudaMemcpyAsync(d_addr, addr.data(), (size_t)n * sizeof(void *), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = od::launch_read_cells(static_cast<const double *const *>(d_addr), n, static_cast<double *>(d_out),
-                                  c->stream);
+                                  c->d_fmt, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(out, d_out, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1093,11 +1124,11 @@ od_status od_read(od_ctx *c, double *dst, int32_t dst_is_device) {
     double *mapped = dst_is_device ? nullptr : device_view(dst);
     if (dst_is_device || mapped) {
         OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, dst_is_device ? dst : mapped,
-                                  c->stream));
+                                  c->d_fmt, c->stream));
     } else {
         s = ensure_stage(c);
         if (s != OD_OK) return s;
-        OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, c->d_stage, c->stream));
+        OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, c->d_stage, c->d_fmt, c->stream));
         OD_CUDA(cudaMemcpyAsync(dst, c->d_stage, (size_t)p.cells * sizeof(double), cudaMemcpyDeviceToHost,
                                 c->stream));
     }
@@ -1122,7 +1153,8 @@ od_status od_write(od_ctx *c, const double *src, int32_t src_is_device) {
                                 c->stream));
         g = c->d_stage;
     }
-    OD_CUDA(od::launch_scatter(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, p.nz, g, c->d_vmax, c->stream));
+    OD_CUDA(od::launch_scatter(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, p.nz, g, c->d_vmax, c->d_fmt, c->words,
+                               c->stream));
     c->ghosts_current = false;  // the scatter writes interiors only
     if (!src_is_device) OD_CUDA(cudaStreamSynchronize(c->stream));
     return OD_OK;
@@ -1138,7 +1170,7 @@ od_status od_write_async(od_ctx *c, const double *src) {
     const od::Plan &p = c->plan;
     OD_CUDA(cudaMemcpyAsync(c->d_stage, src, (size_t)p.cells * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     OD_CUDA(od::launch_scatter(c->d_ch, (int)p.ch.size(), (int)(c->steps & 1), p.nx, p.ny, p.nz, c->d_stage,
-                               c->d_vmax, c->stream));
+                               c->d_vmax, c->d_fmt, c->words, c->stream));
     c->ghosts_current = false;  // interiors only
     return OD_OK;
 }
@@ -1156,7 +1188,7 @@ od_status od_read_async(od_ctx *c, double *dst) {
         OD_CUDA(cudaEventCreateWithFlags(&c->ev_copied, cudaEventDisableTiming));
     }
     const od::Plan &p = c->plan;
-    OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), (int)(c->steps & 1), p.nx, p.ny, c->d_stage, c->stream));
+    OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), (int)(c->steps & 1), p.nx, p.ny, c->d_stage, c->d_fmt, c->stream));
     OD_CUDA(cudaEventRecord(c->ev_gathered, c->stream));
     OD_CUDA(cudaStreamWaitEvent(c->copy_stream, c->ev_gathered, 0));
     OD_CUDA(cudaMemcpyAsync(dst, c->d_stage, (size_t)p.cells * sizeof(double), cudaMemcpyDeviceToHost,
@@ -1181,12 +1213,19 @@ od_status od_face_copy(od_ctx *c, int32_t face, int32_t dir, double *buf, int32_
     DeviceGuard dg(c->device);
     const int par = (int)(c->steps & 1);
     const int nch = (int)p.ch.size();
+    if (dir == 1 && c->words) {
+        // values from outside may exceed the field's own largest, which its
+        // words rely on: from here on the context holds plain doubles
+        OD_CUDA(od::launch_plain(c->d_ch, nch, c->d_fmt, c->stream));
+        c->words = false;
+        drop_graphs(c);  // captured with the kernels over words
+    }
     if (buf_is_device) {
-        OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, buf, p.nx, p.ny, p.nz, c->stream));
+        OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, buf, p.nx, p.ny, p.nz, c->d_fmt, c->stream));
         return OD_OK;
     }
     if (double *mapped = device_view(buf)) {  // pinned host memory: in place
-        OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, mapped, p.nx, p.ny, p.nz, c->stream));
+        OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, mapped, p.nx, p.ny, p.nz, c->d_fmt, c->stream));
         OD_CUDA(cudaStreamSynchronize(c->stream));
         return OD_OK;
     }
@@ -1194,7 +1233,7 @@ od_status od_face_copy(od_ctx *c, int32_t face, int32_t dir, double *buf, int32_
     if (s != OD_OK) return s;
     if (dir == 1)
         OD_CUDA(cudaMemcpyAsync(c->d_stage, buf, (size_t)n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, c->d_stage, p.nx, p.ny, p.nz, c->stream));
+    OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, c->d_stage, p.nx, p.ny, p.nz, c->d_fmt, c->stream));
     if (dir == 0)
         OD_CUDA(cudaMemcpyAsync(buf, c->d_stage, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     OD_CUDA(cudaStreamSynchronize(c->stream));

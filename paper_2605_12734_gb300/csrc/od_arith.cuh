@@ -553,6 +553,163 @@ OD_HD uint32_t anchor_for(uint64_t vmax, int nf) {
     return (uint32_t)e0;
 }
 
+// ---------------------------------------------------------------- fixed-point field words
+//
+// The anchored window pays for turning every operand of every update into its
+// window integer and the quotient back into a double: with six operands that
+// is a third of the update's instructions, and the FP64 adds that avoid part
+// of it run on the scarce FP64 pipe.  A field that is iterated in place need
+// not leave the window at all: its cells can be stored as the window integers
+// themselves.  With a base exponent E0, the word of a double x is
+//   * F = m << (e - E0), its value in units of 2^(E0-1075), when its biased
+//     exponent e lies in [E0, E0+7] (m its 53-bit significand): below 2^60,
+//     so the word's top four bits are zero;
+//   * 0 when x is +0 (also its value in those units);
+//   * otherwise x's own bit pattern, whose top four bits are not all zero,
+//     except for a positive x below 2^-767 outside the window (biased exponent
+//     0..255), whose exponent field is raised by kFxTiny into 1790..2045.
+// The map is one to one as long as the field holds no positive value of
+// exponent 1790 or more; fx_anchor refuses (0) a field that comes near it, and
+// by the maximum principle a Jacobi sweep does not raise a field's largest
+// value beyond its rounding.  An update whose operands are all window words
+// (or zeros) is then integer adds and roundings only; the others decode, use
+// the IEEE operations and encode.
+
+constexpr uint32_t kFxEnd = 0x10000000u;  // a window word's high half is below this
+constexpr uint32_t kFxTiny = 1790u;       // exponent offset of the tiny positives outside the window
+constexpr uint32_t kFxMaxExp = 1779u;     // largest exponent of a field that is kept as words
+
+// The base exponent for a field whose largest value has bit pattern vmax: the
+// window's top binade holds it.  0: the field stays in plain doubles.
+OD_HD uint32_t fx_anchor(uint64_t vmax) {
+    const uint32_t emax = (uint32_t)(vmax >> 52) & 0x7FFu;
+    if (emax > kFxMaxExp) return 0u;
+    return emax > 8u ? emax - 7u : 1u;
+}
+
+// Word of x, and x of a word, for base exponent E0 >= 1; E0 = 0 stands for
+// plain doubles.
+OD_HD uint64_t fx_encode(double x, uint32_t E0) {
+    const uint64_t b = f64_bits(x);
+    const uint32_t hi = (uint32_t)(b >> 32), sh = (hi >> 20) - E0;  // a negative x reads as exponent >= 2048
+    if (E0 == 0u) return b;
+    if (sh <= 7u) return shl31((b & kFrac) | kHid, sh);
+    if (b == 0u || hi >= kFxEnd) return b;
+    return b + ((uint64_t)kFxTiny << 52);
+}
+
+OD_HD double fx_decode(uint64_t w, uint32_t E0) {
+    const uint32_t hi = (uint32_t)(w >> 32);
+    if (E0 == 0u || w == 0u) return f64_from(w);
+    if (hi < kFxEnd) {
+        const uint32_t d = 11u - clz32(hi);  // 0..7 for a window word
+        return f64_from(((uint64_t)(E0 + d - 1u) << 52) + shr31(w, d));
+    }
+    if ((hi >> 20) - kFxTiny <= 255u) return f64_from(w - ((uint64_t)kFxTiny << 52));
+    return f64_from(w);
+}
+
+// Position of the top set bit of x (0xFFFFFFFF for 0)
+OD_HD uint32_t top_bit(uint32_t x) {
+#if defined(__CUDA_ARCH__)
+    uint32_t r;
+    asm("bfind.u32 %0, %1;" : "=r"(r) : "r"(x));
+    return r;
+#else
+    return x ? 31u - (uint32_t)__builtin_clz(x) : 0xFFFFFFFFu;
+#endif
+}
+
+OD_HD uint32_t mulhi32(uint32_t a, uint32_t b) {
+#if defined(__CUDA_ARCH__)
+    return __umulhi(a, b);
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+#endif
+}
+
+// high word of (hi:lo) << (n mod 32)
+OD_HD uint32_t shf_left(uint32_t hi, uint32_t lo, uint32_t n) {
+#if defined(__CUDA_ARCH__)
+    return __funnelshift_l(lo, hi, n);
+#else
+    n &= 31u;
+    return n ? (hi << n) | (lo >> (32u - n)) : hi;
+#endif
+}
+
+// F rounded to 53 significant bits (nearest even) as the sum of its part
+// above the low 23 bits and a second term z (below 2^24), which the next
+// add takes as a third addend.  As in round_acc one binary32 add does the
+// rounding, here of the subnormal binary32 number whose bit pattern is the
+// low 23 bits themselves: with F's top set bit at 52 + d, adding 2^(23+d)
+// units (the binary32 number of exponent field d + 1) rounds to a multiple of
+// 2^d, and subtracting it again leaves the rounded integer as a bit pattern,
+// so nothing is converted.  For F = 0 the addend is finite and x = 0, so the
+// result is 0.
+struct FxRounded {
+    uint64_t a;
+    uint32_t z;
+};
+
+OD_HD FxRounded fx_round(uint64_t F) {
+    const uint32_t c = mad_lo(top_bit((uint32_t)(F >> 32)), 1u << 23, 0u - (19u << 23));
+    FxRounded r;
+    r.z = f32_bits(f32_add_sub(f32_from((uint32_t)F & 0x007FFFFFu), f32_from(c)));
+    r.a = F & ~(uint64_t)0x007FFFFFu;
+    return r;
+}
+
+// F/6 rounded to 53 significant bits, in the same units, for F a sum as
+// fx_round left it (at most 6 * 2^60).  F/6 >= 2^52 has its top bit at 52 + q
+// with q = top_bit(floor(F_hi/6)) - 20 (6 * 2^(52+q) has a zero low word, so
+// the high word decides the binade), and the rounded quotient is
+// floor((F + 2^(q+1)) / 6) with its low q bits cleared: the exact quotient is
+// never a rounding tie (F/6 = 2^q * N/3 with N an integer, see div6), so
+// adding half of the last place and truncating rounds to nearest.  The
+// division works word by word: F_hi = 6 qh + r, and the low word of the
+// quotient is floor((r 2^32 + F_lo + 2^(q+1)) / 6), where F_lo + 2^(q+1) does
+// not carry (F is a multiple of 2^(q+2)) and every term is even.  qh = 0 only
+// for F = 0; qh in [1, 2^20) means that the quotient lies below the window.
+OD_HD uint64_t fx_div6(uint64_t F, uint32_t &qh) {
+    const uint32_t hi = (uint32_t)(F >> 32), lo = (uint32_t)F;
+    qh = mulhi32(hi, 0x2AAAAAABu);  // floor(hi/6) for hi < 2^31
+    const uint32_t t = top_bit(qh);
+    const uint32_t half = shf_left(0x1000u, 0x1000u, t);         // 2^q, q = t - 20
+    const uint32_t keep = shf_left(0xFFFFFFFFu, 0u, t + 12u);    // clears the low q bits
+    const uint32_t r = hi - 6u * qh;
+    const uint32_t v = (lo >> 1) + half + 2u * r;                // (r 2^32 + lo + 2^(q+1)) / 2 less r (2^31 - 2)
+    const uint32_t ql = (mulhi32(v, 0xAAAAAAABu) >> 1) + r * 0x2AAAAAAAu;  // floor(v/3) + r (2^32 - 4)/6
+    return ((uint64_t)qh << 32) | (ql & keep);
+}
+
+// The 3D update of six words; ok = false when an operand or the quotient is
+// not a window word or zero (the result is then meaningless).
+OD_HD uint64_t fx_update3(uint64_t W, uint64_t E, uint64_t S, uint64_t N, uint64_t D, uint64_t U, bool &ok) {
+    const uint32_t any = (uint32_t)((W | E | S) >> 32) | (uint32_t)((N | D | U) >> 32);
+    FxRounded f = fx_round(W + E);
+    f = fx_round(f.a + f.z + S);
+    f = fx_round(f.a + f.z + N);
+    f = fx_round(f.a + f.z + D);
+    f = fx_round(f.a + f.z + U);
+    uint32_t qh;
+    const uint64_t Q = fx_div6(f.a + f.z, qh);
+    ok = (any < kFxEnd) & (qh - 1u >= (1u << 20) - 1u);
+    return Q;
+}
+
+// The 2D update of four words: the division by 4 is a shift (exact when the
+// quotient lies in the window).
+OD_HD uint64_t fx_update2(uint64_t W, uint64_t E, uint64_t S, uint64_t N, bool &ok) {
+    const uint32_t any = (uint32_t)((W | E) >> 32) | (uint32_t)((S | N) >> 32);
+    FxRounded f = fx_round(W + E);
+    f = fx_round(f.a + f.z + S);
+    f = fx_round(f.a + f.z + N);
+    const uint64_t Q = (f.a + f.z) >> 2;
+    ok = (any < kFxEnd) & ((uint32_t)(Q >> 32) - 1u >= (1u << 20) - 1u);
+    return Q;
+}
+
 // ---------------------------------------------------------------- update
 
 // s / 6 on the integer pipes without a branch; ok = false when s is outside

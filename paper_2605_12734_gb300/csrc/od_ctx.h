@@ -16,6 +16,7 @@ struct od_ctx {
     od::Plan plan;
     int device = 0;
     int num_sms = 0;
+    int resident = 0;                 // CTAs of the fused step over words that the GPU holds at once
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     char *arena = nullptr;
@@ -25,7 +26,11 @@ struct od_ctx {
     ErrDev *d_err = nullptr;
     int32_t *d_queue = nullptr, *d_epoch = nullptr, *d_dep_ptr = nullptr, *d_dep_idx = nullptr,
             *d_order = nullptr;
+    TileRec *d_rec = nullptr;         // tiles as the sweep over words reads them
     uint64_t *d_vmax = nullptr;       // largest value of the field (bits), in the arena's queue block
+    FmtDev *d_fmt = nullptr;          // format of the field's words, beside it
+    bool words = false;               // the field may be kept as fixed-point words (the default
+                                      // arithmetic, until a face is fed from outside)
     bool ghosts_current = true;       // internal ghost layers of the current parity hold the
                                       // neighbours' faces (false after a fused step or an import)
     std::vector<ChareDev> h_ch;       // host copy (device pointers)
@@ -55,6 +60,8 @@ struct od_ctx {
     // one step from each parity
     cudaGraphExec_t gf = nullptr, gf1[2] = {nullptr, nullptr};
     int64_t g2_kernels = 0, g1_kernels[2] = {0, 0};
+    // arithmetic mode the tile kernels are launched in
+    int kernel_mode() const { return od::kernel_mode(plan.amode, words); }
     int64_t g2_calls = 0, g1_calls[2] = {0, 0};
 };
 

@@ -65,12 +65,44 @@ struct TileDev {
     int32_t pad;
 };
 
+// One compute task as the sweep over fixed-point words reads it: everything
+// about the tile in one 256-byte record (one coalesced load by a warp) instead
+// of a chain of dependent loads through the tile, chare, neighbour and
+// dependency tables.  Built on the device once per context.  Pointers come in
+// both parities; a face without a neighbour, or that the tile does not touch,
+// is null.
+struct alignas(256) TileRec {
+    double *own[2];          // the tile's first copied row (2D: cell) of plane -1
+    const double *xlo[2];    // the x neighbours' boundary column: first row of the tile, plane -1
+    const double *xhi[2];
+    const double *ylo[2];    // the y neighbours' boundary row next to the tile, plane -1
+    const double *yhi[2];
+    const double *zlo[2];    // the z neighbours' boundary plane, the tile's rows
+    const double *zhi[2];
+    int32_t bx, pitch, plane;           // row cells; doubles per row, per plane
+    int32_t rows, cells;                // rows of the tile (1 in 2D), cells of a plane of it
+    int32_t k0, nk, bz;                 // planes computed, planes of the chare
+    int32_t xlo_pitch, xlo_plane, xhi_pitch, xhi_plane, ylo_plane, yhi_plane;
+    int32_t run;             // bytes of a plane's copy
+    int32_t ndep;            // tiles whose previous step it waits for
+    int32_t dep[20];         // their indices; more than 20: dep[0] is their place in dep_idx
+};
+static_assert(sizeof(TileRec) == 256, "one load of 8 bytes per lane");
+
 // Error record written by kernels (first error wins).
 struct ErrDev {
     int32_t code;
     int32_t tile;
     int32_t step;
     int32_t pad[13];
+};
+
+// How a context's arrays hold the field (device words beside the ticket
+// counter): base = 0 plain doubles, else the base exponent of its fixed-point
+// words (od_arith.cuh).  done counts the blocks of a change of format.
+struct FmtDev {
+    uint32_t base;
+    uint32_t done;
 };
 
 // Arguments of the tile kernels (passed by value).
@@ -82,10 +114,14 @@ struct KArgs {
     int32_t *epoch;          // persistent: steps finished per tile in this launch
     const int32_t *dep_ptr;  // persistent: CSR of the tiles each tile reads
     const int32_t *dep_idx;
-    const int32_t *order;    // persistent: tile of each queue position
+    const int32_t *order;    // persistent: tile of each queue position (null: in index order,
+                             // sweep over words only)
     const uint64_t *vmax;    // bit pattern of the largest value the field holds (a positive
                              // double), from which the anchored arithmetic takes its window
-    int32_t tile_begin;      // static launch: tile of blockIdx.x == 0
+    const FmtDev *fmt;       // format of the field's words
+    const TileRec *rec;      // the tiles as the sweep over words reads them
+    int32_t tile_begin;      // static launch: its first tile
+    int32_t tile_count;      // static launch: its tiles
     int32_t ntiles;          // tiles per step
     int32_t parity;          // static launch: parity of the source buffer
     int32_t iters;           // persistent: steps in this launch

@@ -29,6 +29,7 @@ void *tile_kernel_am12(int threads, int cpt, int kind);
 void *tile_kernel_am13(int threads, int cpt, int kind);
 void *tile_kernel_am14(int threads, int cpt, int kind);
 void *tile_kernel_am15(int threads, int cpt, int kind);
+void *tile_kernel_am16(int threads, int cpt, int kind);
 void *tile_kernel2d_am0(int threads, int cpt, int kind);
 void *tile_kernel2d_am1(int threads, int cpt, int kind);
 void *tile_kernel2d_am2(int threads, int cpt, int kind);
@@ -43,6 +44,7 @@ void *tile_kernel2d_am12(int threads, int cpt, int kind);
 void *tile_kernel2d_am13(int threads, int cpt, int kind);
 void *tile_kernel2d_am14(int threads, int cpt, int kind);
 void *tile_kernel2d_am15(int threads, int cpt, int kind);
+void *tile_kernel2d_am16(int threads, int cpt, int kind);
 
 namespace {
 
@@ -64,6 +66,7 @@ void *tile_kernel(int stencil, int amode, int threads, int cpt, int kind) {
         case 13: return tile_kernel2d_am13(threads, cpt, kind);
         case 14: return tile_kernel2d_am14(threads, cpt, kind);
         case 15: return tile_kernel2d_am15(threads, cpt, kind);
+        case 16: return tile_kernel2d_am16(threads, cpt, kind);
         default: return nullptr;
     }
     if (stencil != OD_STENCIL_3D7) return nullptr;
@@ -84,6 +87,7 @@ void *tile_kernel(int stencil, int amode, int threads, int cpt, int kind) {
         case 13: return tile_kernel_am13(threads, cpt, kind);
         case 14: return tile_kernel_am14(threads, cpt, kind);
         case 15: return tile_kernel_am15(threads, cpt, kind);
+        case 16: return tile_kernel_am16(threads, cpt, kind);
         default: return nullptr;
     }
 }
@@ -114,7 +118,7 @@ __device__ __forceinline__ double field_init(int64_t gx, int64_t gy, int64_t gz,
 // 2D padded index gx + (nx+2)*gz; (ox, oy, oz) is a shard's offset in the
 // global grid nx x ny x nz.
 __global__ void k_init(const ChareDev *ch, int nch, int64_t nx, int64_t ny, int64_t nz, int64_t ox, int64_t oy,
-                       int64_t oz, uint64_t seed, int mode, int stencil) {
+                       int64_t oz, uint64_t seed, int mode, int stencil, uint32_t base) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int c = blockIdx.y; c < nch; c += gridDim.y) {
         const ChareDev &C = ch[c];
@@ -136,10 +140,65 @@ __global__ void k_init(const ChareDev *ch, int nch, int64_t nx, int64_t ny, int6
                         v = field_init(gx, gy, gz, nx, ny, nz, seed, mode);
                     }
                 }
+                v = f64_from(fx_encode(v, base));
                 a0[cp] = v;
                 a1[cp] = v;
             }
         }
+    }
+}
+
+// One thread per tile: its record (see TileRec) from the tables.
+__global__ void k_tile_recs(const ChareDev *ch, const TileDev *tiles, int64_t ntiles, const int32_t *dep_ptr,
+                            const int32_t *dep_idx, TileRec *rec, int stencil) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntiles;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const TileDev T = tiles[t];
+        const ChareDev &C = ch[T.c];
+        const bool d3 = stencil == OD_STENCIL_3D7;
+        TileRec R;
+        R.bx = C.bx;
+        R.pitch = C.pitch;
+        R.plane = C.rows * C.pitch;
+        R.rows = d3 ? T.nj : 1;
+        R.cells = d3 ? T.nj * C.bx : T.ni;
+        R.k0 = T.k0;
+        R.nk = T.nk;
+        R.bz = C.bz;
+        R.run = d3 ? (T.nj + 2) * C.pitch * 8 : ((T.ni + 3) & ~1) * 8;
+        const bool low = T.k0 == 0, high = T.k0 + T.nk >= C.bz;  // touches the chare's z faces
+        const int64_t org = d3 ? (int64_t)T.j0 * C.pitch : T.i0;
+        const ChareDev *N[6];
+        for (int f = 0; f < 6; ++f) N[f] = C.nbr[f] >= 0 ? &ch[C.nbr[f]] : nullptr;
+        const ChareDev *X0 = N[OD_FACE_XLO], *X1 = N[OD_FACE_XHI], *Y0 = N[OD_FACE_YLO], *Y1 = N[OD_FACE_YHI],
+                       *Z0 = N[OD_FACE_ZLO], *Z1 = N[OD_FACE_ZHI];
+        if (!d3 && T.i0 != 0) X0 = nullptr;
+        if (!d3 && T.i0 + T.ni != C.bx) X1 = nullptr;
+        if (!d3 || T.j0 != 0) Y0 = nullptr;
+        if (!d3 || T.j0 + T.nj != C.by) Y1 = nullptr;
+        if (!low) Z0 = nullptr;
+        if (!high) Z1 = nullptr;
+        for (int p = 0; p < 2; ++p) {
+            R.own[p] = C.A[p] + org;
+            // y- and z-neighbours share the chare's x extent, so its pitch;
+            // z-neighbours its y extent too, so its plane
+            R.xlo[p] = X0 ? X0->A[p] + X0->bx + (d3 ? (int64_t)(T.j0 + 1) * X0->pitch : 0) : nullptr;
+            R.xhi[p] = X1 ? X1->A[p] + 1 + (d3 ? (int64_t)(T.j0 + 1) * X1->pitch : 0) : nullptr;
+            R.ylo[p] = Y0 ? Y0->A[p] + (int64_t)Y0->by * C.pitch : nullptr;
+            R.yhi[p] = Y1 ? Y1->A[p] + C.pitch : nullptr;
+            R.zlo[p] = Z0 ? Z0->A[p] + (int64_t)Z0->bz * R.plane + org : nullptr;
+            R.zhi[p] = Z1 ? Z1->A[p] + R.plane + org : nullptr;
+        }
+        R.xlo_pitch = X0 ? X0->pitch : 0;
+        R.xlo_plane = X0 ? X0->rows * X0->pitch : 0;
+        R.xhi_pitch = X1 ? X1->pitch : 0;
+        R.xhi_plane = X1 ? X1->rows * X1->pitch : 0;
+        R.ylo_plane = Y0 ? Y0->rows * C.pitch : 0;
+        R.yhi_plane = Y1 ? Y1->rows * C.pitch : 0;
+        const int32_t q0 = dep_ptr[t];
+        R.ndep = dep_ptr[t + 1] - q0;
+        for (int d = 0; d < 20; ++d) R.dep[d] = R.ndep > 20 ? q0 : d < R.ndep ? dep_idx[q0 + d] : 0;
+        rec[t] = R;
     }
 }
 
@@ -215,7 +274,8 @@ __global__ void k_ghost_refresh(const ChareDev *ch, int nch, int p) {
 // dense: x faces nz x ny (y fastest), y faces nz x nx, z faces ny x nx (x
 // fastest).
 __global__ void k_face_copy(const ChareDev *ch, int nch, int p, int f, int dir, double *buf, int64_t nx, int64_t ny,
-                            int64_t nz) {
+                            int64_t nz, const FmtDev *fmt) {
+    const uint32_t base = fmt->base;
     for (int c = blockIdx.y; c < nch; c += gridDim.y) {
         const ChareDev &C = ch[c];
         const bool on_face = f == OD_FACE_XLO ? C.x0 == 0 : f == OD_FACE_XHI ? C.x0 + C.bx == nx
@@ -231,16 +291,17 @@ __global__ void k_face_copy(const ChareDev *ch, int nch, int p, int f, int dir, 
             else if (f < 4) g = (C.z0 + b) * nx + C.x0 + a;
             else g = (C.y0 + b) * nx + C.x0 + a;
             const int64_t o = face_offset(C, f, q, dir != 0);
-            if (dir == 0) buf[g] = C.A[p][o];
-            else C.A[p][o] = buf[g];
+            if (dir == 0) buf[g] = fx_decode(f64_bits(C.A[p][o]), base);
+            else C.A[p][o] = f64_from(fx_encode(buf[g], base));
         }
     }
 }
 
-// Selected cells: out[i] = *addr[i] (addresses inside the chares' arrays).
-__global__ void k_read_cells(const double *const *addr, int64_t n, double *out) {
+// Selected cells: out[i] = the value at *addr[i] (addresses inside the chares' arrays).
+__global__ void k_read_cells(const double *const *addr, int64_t n, double *out, const FmtDev *fmt) {
+    const uint32_t base = fmt->base;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = *addr[i];
+        out[i] = fx_decode(f64_bits(*addr[i]), base);
 }
 
 // Rows a warp moves per pass of the gather and scatter: the loads of all of
@@ -252,7 +313,8 @@ constexpr int kIoRows = 4;
 // A11: interiors of parity p -> global x-fastest array.  Each warp moves
 // kIoRows interior rows per pass (coalesced on both sides), one 32-bit
 // division per row.
-__global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, double *g) {
+__global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, double *g, const FmtDev *fmt) {
+    const uint32_t base = fmt->base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int c = blockIdx.y; c < nch; c += gridDim.y) {
         const ChareDev &C = ch[c];
@@ -273,7 +335,8 @@ __global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t
 #pragma unroll
                 for (int u = 0; u < kIoRows; ++u) v[u] = src[u][i];
 #pragma unroll
-                for (int u = 0; u < kIoRows; ++u) dst[u][i] = v[u];  // a repeated row stores the same value
+                for (int u = 0; u < kIoRows; ++u)
+                    dst[u][i] = fx_decode(f64_bits(v[u]), base);  // a repeated row stores the same value
             }
         }
     }
@@ -290,7 +353,8 @@ __global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t
 // which anchors the exact arithmetic's window (od_arith.cuh); at most one
 // atomic per warp.
 __global__ void k_scatter(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, int64_t nz,
-                          const double *g, unsigned long long *vmax) {
+                          const double *g, unsigned long long *vmax, const FmtDev *fmt) {
+    const uint32_t base = fmt->base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     unsigned long long vm = 0;
     for (int c = blockIdx.y; c < nch; c += gridDim.y) {
@@ -313,7 +377,7 @@ __global__ void k_scatter(const ChareDev *ch, int nch, int p, int64_t nx, int64_
                 for (int u = 0; u < kIoRows; ++u) v[u] = src[u][i];
 #pragma unroll
                 for (int u = 0; u < kIoRows; ++u) {
-                    dst[u][i] = v[u];  // a repeated row stores the same value
+                    dst[u][i] = f64_from(fx_encode(v[u], base));  // a repeated row stores the same value
                     const unsigned long long b = (unsigned long long)__double_as_longlong(v[u]);
                     if (b < 0x7FF0000000000000ull && b > vm) vm = b;  // positive and finite
                 }
@@ -329,6 +393,65 @@ __global__ void k_scatter(const ChareDev *ch, int nch, int p, int64_t nx, int64_
     // the word only grows: a warp whose maximum is not above it skips the
     // atomic (a field within the initial bound [0, 1) then issues none)
     if (lane == 0 && vm != 0 && vmax && vm > *(volatile unsigned long long *)vmax) atomicMax(vmax, vm);
+}
+
+// After an import: the field's largest value may have outgrown the format it
+// was written in.  If it has (every block finds the same answer: nothing else
+// writes these words), the whole field takes the format that its largest
+// value asks for: the interiors of parity p from the import's source again,
+// every ghost cell of both parities (the Dirichlet shell among them) from its
+// present words; the other parity's interiors are written before they are
+// read.  The last block records the format.  A field that stayed within its
+// format costs one launch that reads two words.
+__global__ void k_refit(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, const double *g,
+                        const unsigned long long *vmax, FmtDev *fmt) {
+    const uint32_t from = fmt->base;
+    if (from == 0u) return;  // plain doubles hold every field
+    const uint32_t to = fx_anchor(*vmax);
+    if (to == from) return;
+    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    const int64_t wid = (int64_t)blockIdx.x * nwarps + (threadIdx.x >> 5), nw = (int64_t)gridDim.x * nwarps;
+    for (int c = 0; c < nch; ++c) {
+        const ChareDev &C = ch[c];
+        const int nrow = C.rows * (C.bz + 2);
+        for (int rr = (int)((wid + c) % nw); rr < nrow; rr += (int)nw) {
+            const int kp = rr / C.rows, rp = rr - kp * C.rows;
+            const int j = rp - C.row0, k = kp - 1;
+            const bool inside = j >= 0 && j < C.by && k >= 0 && k < C.bz;
+            double *a = C.A[p] + (int64_t)rr * C.pitch, *b = C.A[p ^ 1] + (int64_t)rr * C.pitch;
+            for (int cp = lane; cp < C.pitch; cp += 32) {
+                if (inside && cp >= 1 && cp <= C.bx) {
+                    a[cp] = f64_from(fx_encode(g[((C.z0 + k) * ny + C.y0 + j) * nx + C.x0 + cp - 1], to));
+                } else {
+                    a[cp] = f64_from(fx_encode(fx_decode(f64_bits(a[cp]), from), to));
+                    b[cp] = f64_from(fx_encode(fx_decode(f64_bits(b[cp]), from), to));
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&fmt->done, 1u) == gridDim.x - 1u) {
+            fmt->done = 0u;
+            fmt->base = to;
+        }
+    }
+}
+
+// Every word of both parities to plain doubles (the caller clears the format
+// word behind it).
+__global__ void k_plain(const ChareDev *ch, int nch, const FmtDev *fmt) {
+    const uint32_t base = fmt->base;
+    if (base == 0u) return;
+    for (int c = blockIdx.y; c < nch; c += gridDim.y) {
+        const ChareDev &C = ch[c];
+        const int64_t n = (int64_t)C.rows * (C.bz + 2) * C.pitch;
+        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+            C.A[0][e] = fx_decode(f64_bits(C.A[0][e]), base);
+            C.A[1][e] = fx_decode(f64_bits(C.A[1][e]), base);
+        }
+    }
 }
 
 // Arithmetic self-test: op 0 div6, 1 add (integer pipes); 2 division by 6,
@@ -392,13 +515,21 @@ cudaError_t prepare_tile_kernels(int threads, int cpt, int amode, int smem_bytes
     return cudaSuccess;
 }
 
-cudaError_t launch_tiles(const KArgs &a, int grid, int threads, int cpt, int amode, bool push, int smem_bytes,
-                         cudaStream_t s) {
-    void *f = tile_kernel(a.stencil, amode, threads, cpt, push ? 1 : 0);
+// The kernels over fixed-point words (mode 16, kinds 0..2) have a producer
+// warp beside their compute threads.
+static int block_threads(int amode, int threads) { return amode == 16 ? threads + 32 : threads; }
+
+cudaError_t launch_tiles(const KArgs &a0, int tiles, int threads, int cpt, int amode, bool push, int smem_bytes,
+                         int resident, cudaStream_t s) {
+    void *f = tile_kernel(a0.stencil, amode, threads, cpt, push ? 1 : 0);
     if (!f) return cudaErrorInvalidValue;
-    if (grid <= 0) return cudaSuccess;
+    if (tiles <= 0) return cudaSuccess;
+    KArgs a = a0;
+    a.tile_count = tiles;
+    // those kernels take several tiles per CTA, so no more CTAs than fit at once
+    const int grid = amode == 16 && resident > 0 ? std::min(tiles, resident) : tiles;
     void *args[] = {(void *)&a};
-    return cudaLaunchKernel(f, dim3(grid), dim3(threads), args, (size_t)smem_bytes, s);
+    return cudaLaunchKernel(f, dim3(grid), dim3(block_threads(amode, threads)), args, (size_t)smem_bytes, s);
 }
 
 cudaError_t launch_persistent(const KArgs &a, int grid, int threads, int cpt, int amode, int smem_bytes,
@@ -407,7 +538,7 @@ cudaError_t launch_persistent(const KArgs &a, int grid, int threads, int cpt, in
     if (!f) return cudaErrorInvalidValue;
     if (grid <= 0) return cudaSuccess;
     void *args[] = {(void *)&a};
-    return cudaLaunchKernel(f, dim3(grid), dim3(threads), args, (size_t)smem_bytes, s);
+    return cudaLaunchKernel(f, dim3(grid), dim3(block_threads(amode, threads)), args, (size_t)smem_bytes, s);
 }
 
 cudaError_t launch_tiles_multi(const KArgs *jobs, const int32_t *first, int32_t njobs, const KArgs &geom, int grid,
@@ -440,19 +571,35 @@ cudaError_t persistent_occupancy(int threads, int cpt, int amode, int smem_bytes
                                  int *blocks_per_sm) {
     void *f = tile_kernel(stencil, amode, threads, cpt, 2);
     if (!f) return cudaErrorInvalidValue;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, (size_t)smem_bytes);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, block_threads(amode, threads),
+                                                         (size_t)smem_bytes);
+}
+
+cudaError_t tiles_occupancy(int threads, int cpt, int amode, int smem_bytes, int stencil, int *blocks_per_sm) {
+    void *f = tile_kernel(stencil, amode, threads, cpt, 1);
+    if (!f) return cudaErrorInvalidValue;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, block_threads(amode, threads),
+                                                         (size_t)smem_bytes);
 }
 
 cudaError_t launch_init(const ChareDev *ch, int nch, int64_t gnx, int64_t gny, int64_t gnz, int64_t gx0,
-                        int64_t gy0, int64_t gz0, uint64_t seed, int mode, int stencil, cudaStream_t s) {
+                        int64_t gy0, int64_t gz0, uint64_t seed, int mode, int stencil, uint32_t base,
+                        cudaStream_t s) {
     k_init<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, gnx, gny, gnz, gx0, gy0, gz0, seed, mode,
-                                                                stencil);
+                                                                stencil, base);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tile_recs(const ChareDev *ch, const TileDev *tiles, int64_t ntiles, const int32_t *dep_ptr,
+                             const int32_t *dep_idx, TileRec *rec, int stencil, cudaStream_t s) {
+    const int grid = (int)std::min<int64_t>((ntiles + 127) / 128, 4096);
+    k_tile_recs<<<grid, 128, 0, s>>>(ch, tiles, ntiles, dep_ptr, dep_idx, rec, stencil);
     return cudaGetLastError();
 }
 
 cudaError_t launch_face_copy(const ChareDev *ch, int nch, int parity, int face, int dir, double *buf, int64_t nx,
-                             int64_t ny, int64_t nz, cudaStream_t s) {
-    k_face_copy<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, parity, face, dir, buf, nx, ny, nz);
+                             int64_t ny, int64_t nz, const FmtDev *fmt, cudaStream_t s) {
+    k_face_copy<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, parity, face, dir, buf, nx, ny, nz, fmt);
     return cudaGetLastError();
 }
 
@@ -472,24 +619,34 @@ cudaError_t launch_unpack(const ChareDev *ch, int c, int parity, int slot, int e
     return cudaGetLastError();
 }
 
-cudaError_t launch_read_cells(const double *const *addr, int64_t n, double *out, cudaStream_t s) {
+cudaError_t launch_read_cells(const double *const *addr, int64_t n, double *out, const FmtDev *fmt, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int grid = (int)std::min<int64_t>((n + 255) / 256, 1024);
-    k_read_cells<<<grid, 256, 0, s>>>(addr, n, out);
+    k_read_cells<<<grid, 256, 0, s>>>(addr, n, out, fmt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gather(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, double *g,
-                          cudaStream_t s) {
-    k_gather<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, parity, nx, ny, g);
+                          const FmtDev *fmt, cudaStream_t s) {
+    k_gather<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, parity, nx, ny, g, fmt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scatter(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, int64_t nz,
-                           const double *g, uint64_t *vmax, cudaStream_t s) {
+                           const double *g, uint64_t *vmax, FmtDev *fmt, bool words, cudaStream_t s) {
     k_scatter<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, parity, nx, ny, nz, g,
-                                                                    (unsigned long long *)vmax);
+                                                                    (unsigned long long *)vmax, fmt);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || !words) return e;
+    k_refit<<<608, 256, 0, s>>>(ch, nch, parity, nx, ny, g, (const unsigned long long *)vmax, fmt);
     return cudaGetLastError();
+}
+
+cudaError_t launch_plain(const ChareDev *ch, int nch, FmtDev *fmt, cudaStream_t s) {
+    k_plain<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, fmt);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return cudaMemsetAsync(fmt, 0, sizeof *fmt, s);
 }
 
 cudaError_t launch_ghost_refresh(const ChareDev *ch, int nch, int parity, cudaStream_t s) {

@@ -8,18 +8,21 @@
 namespace od {
 
 // Tile kernels exist for (threads, cells per thread) in {128}x{2,4,8},
-// {256}x{1,2,4,8}, {512}x{1,2}, arithmetic modes 0..15 and both stencils
+// {256}x{1,2,4,8}, {512}x{1,2}, arithmetic modes 0..15 (and 16, mode 12 over
+// fixed-point field words) and both stencils
 // (OD_STENCIL_3D7, OD_STENCIL_2D5) (od_tile.cuh).
 bool tile_shape_supported(int threads, int cpt, int amode, int stencil);
 
 // Raise the dynamic shared-memory limit of the tile kernels of one shape.
 cudaError_t prepare_tile_kernels(int threads, int cpt, int amode, int smem_bytes, int stencil);
 
-// One CTA per tile, tiles [a.tile_begin, a.tile_begin + grid), of stencil
-// a.stencil (so for launch_persistent).  push = 1 also
-// stores each new boundary value into the neighbour's ghost layer.
-cudaError_t launch_tiles(const KArgs &a, int grid, int threads, int cpt, int amode, bool push, int smem_bytes,
-                         cudaStream_t s);
+// The tiles [a.tile_begin, a.tile_begin + tiles) of stencil a.stencil (so for
+// launch_persistent), one CTA per tile; the kernels over fixed-point words
+// take several tiles per CTA when there are more than `resident` CTAs (what
+// the GPU holds at once; 0: one per tile).  push = 1: a fused step, whose
+// tiles read the faces of their neighbours' arrays.
+cudaError_t launch_tiles(const KArgs &a, int tiles, int threads, int cpt, int amode, bool push, int smem_bytes,
+                         int resident, cudaStream_t s);
 
 // One fused step of several jobs (continuous batching): jobs[j] (device
 // array) is job j's KArgs with its source parity, first[j] its first block
@@ -42,30 +45,43 @@ cudaError_t launch_persistent(const KArgs &a, int grid, int threads, int cpt, in
                               cudaStream_t s);
 cudaError_t persistent_occupancy(int threads, int cpt, int amode, int smem_bytes, int stencil,
                                  int *blocks_per_sm);
+cudaError_t tiles_occupancy(int threads, int cpt, int amode, int smem_bytes, int stencil, int *blocks_per_sm);
 cudaError_t persistent_multi_occupancy(int threads, int cpt, int amode, int smem_bytes, int stencil,
                                        int *blocks_per_sm);
 
-// The initial field of a shard at offset (gx0, gy0, gz0) of a global grid
+// The tiles' records for the sweep over words, from the tables (TileRec).
+cudaError_t launch_tile_recs(const ChareDev *ch, const TileDev *tiles, int64_t ntiles, const int32_t *dep_ptr,
+                             const int32_t *dep_idx, TileRec *rec, int stencil, cudaStream_t s);
+
+// Every call below that moves field values between a context's arrays and a
+// buffer of doubles takes the context's format word (FmtDev).
+
+// The initial field, written in format `base` (0: plain doubles), of a shard at offset (gx0, gy0, gz0) of a global grid
 // gnx x gny x gnz (the whole grid: offsets 0, global = local extents).
 cudaError_t launch_init(const ChareDev *ch, int nch, int64_t gnx, int64_t gny, int64_t gnz, int64_t gx0,
-                        int64_t gy0, int64_t gz0, uint64_t seed, int mode, int stencil, cudaStream_t s);
+                        int64_t gy0, int64_t gz0, uint64_t seed, int mode, int stencil, uint32_t base,
+                        cudaStream_t s);
 // Domain-face exchange of a shard (od_face_copy): dir 0 copies the boundary
 // layer of parity p on face f into buf, dir 1 buf into the ghost layer.
 cudaError_t launch_face_copy(const ChareDev *ch, int nch, int parity, int face, int dir, double *buf, int64_t nx,
-                             int64_t ny, int64_t nz, cudaStream_t s);
+                             int64_t ny, int64_t nz, const FmtDev *fmt, cudaStream_t s);
 cudaError_t launch_pack(const ChareDev *ch, int c, int parity, int elems, cudaStream_t s);
 cudaError_t launch_unpack(const ChareDev *ch, int c, int parity, int slot, int elems, cudaStream_t s);
 // out[i] = *addr[i] for n device addresses (od_read_cells).
-cudaError_t launch_read_cells(const double *const *addr, int64_t n, double *out, cudaStream_t s);
+cudaError_t launch_read_cells(const double *const *addr, int64_t n, double *out, const FmtDev *fmt, cudaStream_t s);
 cudaError_t launch_gather(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, double *g,
-                          cudaStream_t s);
+                          const FmtDev *fmt, cudaStream_t s);
 // Arithmetic self-test over device arrays (op: 0 div6, 1 add on the integer
 // pipes; 2 division by 6, 3 add on the FP64 pipe).
 cudaError_t launch_arith(int op, const double *a, const double *b, double *out, int64_t n, cudaStream_t s);
 // Import (od_write): also raises *vmax (device word, may be null) to the
-// bit pattern of the largest positive finite value written.
+// bit pattern of the largest positive finite value written; words = true
+// (the context may hold fixed-point words): the field then takes a wider
+// format if that value asks for it.
 cudaError_t launch_scatter(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, int64_t nz,
-                           const double *g, uint64_t *vmax, cudaStream_t s);
+                           const double *g, uint64_t *vmax, FmtDev *fmt, bool words, cudaStream_t s);
+// The whole context to plain doubles, for good.
+cudaError_t launch_plain(const ChareDev *ch, int nch, FmtDev *fmt, cudaStream_t s);
 // Internal ghost layers of parity `parity` from the neighbours' boundaries.
 cudaError_t launch_ghost_refresh(const ChareDev *ch, int nch, int parity, cudaStream_t s);
 

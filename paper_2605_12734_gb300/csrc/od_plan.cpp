@@ -18,7 +18,6 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr int32_t kMaxSmem = 232448;  // 227 KB opt-in per CTA on sm_100/sm_103
 constexpr int32_t kSmemHeader = 256;  // mbarriers + neighbour push table
-constexpr int32_t kDefaultArith = 12;  // two FP64 adds, the rest in the anchored integer window
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 int32_t round_up(int32_t v, int32_t a) { return (v + a - 1) / a * a; }
@@ -137,10 +136,9 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     p.stages = cfg->stages ? cfg->stages : 4;
     p.tile_y = cfg->tile_y;
     p.tile_z = cfg->tile_z;
-    // default: the anchored window -- in 3D two FP64 adds and the rest in
-    // the window (202 G updates/s at 512^3 in 4096 chares against 167 for
-    // the earlier tail form), in 2D one FP64 add (279 against 252 for one
-    // per-cell window add at 32768^2)
+    // default: the anchored window, the field kept as words of it (512^3 in
+    // 4096 chares: 267 G updates/s, against 205 with plain doubles and two FP64
+    // adds; 32768^2: 378 against 345 with one)
     p.amode = cfg->arith >= 0 ? cfg->arith : kDefaultArith;
     if (p.amode > 15) {
         *err = "arith must be in [0, 15] (or -1 for the default)";
@@ -401,6 +399,18 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
         *err = "tile too large for the kernels' cell encoding; lower tile_y";
         return OD_EINVAL;
     }
+    // Ring depth of the sweep over words, when none is asked for: its producer
+    // runs ahead as far as the ring goes, so it is as deep as the shared
+    // memory of the CTAs that the registers admit, up to 6 planes (3D; 0.524 ms
+    // a step with 4, 0.500 with 5, 0.489 with 6 at 512^3 in 4096 chares) or 8
+    // rows (2D; 16384^2 0.745 ms with 4, 0.665 with 8); never fewer than the 4
+    // of the other sweeps.
+    if (cfg->stages == 0 && p.amode == kDefaultArith) {
+        const bool d3 = p.stencil == OD_STENCIL_3D7;
+        const int64_t per_cta = 228 * 1024 / words_ctas(p.threads, p.cpt, d3) - 2048 - kSmemHeader;
+        const int64_t fit = per_cta / ((int64_t)p.stage_doubles * 8);
+        p.stages = (int32_t)std::max<int64_t>(4, std::min<int64_t>(d3 ? 6 : 8, fit));
+    }
     int64_t smem = kSmemHeader + (int64_t)p.stages * p.stage_doubles * 8;
     if (smem > kMaxSmem) {
         char buf[200];
@@ -486,6 +496,7 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     p.off_dep_ptr = take(p.dep_ptr.size() * sizeof(int32_t));
     p.off_dep_idx = take(std::max<size_t>(1, p.dep_idx.size()) * sizeof(int32_t));
     p.off_order = take(p.order.size() * sizeof(int32_t));
+    p.off_rec = take(p.amode == kDefaultArith ? p.tiles.size() * sizeof(TileRec) : 0);
     for (auto &h : p.ch) {
         size_t a_bytes = (size_t)(h.bz + 2) * (size_t)h.rows * (size_t)h.pitch * 8;
         size_t f_bytes = (size_t)h.foff[6] * 8;

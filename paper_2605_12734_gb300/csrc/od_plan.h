@@ -12,6 +12,20 @@
 
 namespace od {
 
+// Default arithmetic: the anchored integer window, with the field kept as
+// fixed-point words where the context allows it (od_arith.cuh).
+constexpr int32_t kDefaultArith = 12;
+constexpr int32_t kFxMode = 16;  // the tile kernels' mode for mode 12 over such words
+// Resident CTAs per SM of the kernels over words (od_words.cuh): their
+// register budget a thread, for NT compute threads and the producer warp.
+// Measured at 512^3 in 4096 chares (128 x 4): 64 registers 0.489 ms a step,
+// 56 (7 CTAs, a few spills) 0.496, 80 (5 CTAs) 0.60; 32768^2: 56 registers.
+constexpr int words_regs(int cpt, bool d3) { return cpt > 4 ? 112 : d3 ? 64 : 56; }
+constexpr int words_ctas(int nt, int cpt, bool d3) {
+    return 65536 / (words_regs(cpt, d3) * (nt + 32)) > 1 ? 65536 / (words_regs(cpt, d3) * (nt + 32)) : 1;
+}
+inline int32_t kernel_mode(int32_t arith, bool words) { return words && arith == kDefaultArith ? kFxMode : arith; }
+
 struct HostChare {
     int32_t cx, cy, cz;
     int64_t x0, y0, z0;
@@ -45,7 +59,7 @@ struct Plan {
     int32_t smem_bytes = 0;                   // dynamic smem per CTA
     // arena layout (byte offsets from the arena base)
     size_t off_err = 0, off_queue = 0, off_epoch = 0, off_chares = 0, off_tiles = 0;
-    size_t off_dep_ptr = 0, off_dep_idx = 0, off_order = 0;
+    size_t off_dep_ptr = 0, off_dep_idx = 0, off_rec = 0, off_order = 0;
     size_t arena_bytes = 0;
     // model
     int64_t cells = 0, face_internal = 0, face_dirichlet = 0;

@@ -194,7 +194,8 @@ od_config job_config(od_server *s, Job *j) {
     c.autotune = 0;
     c.threads = s->threads ? s->threads : j->threads;
     c.cells_per_thread = s->threads ? s->cpt : j->cpt;
-    c.stages = s->stages;
+    // per-job launches leave the ring depth to the planner unless it is given
+    c.stages = s->job_streams.empty() ? s->stages : s->cfg.stages;
     c.arith = s->arith;
     c.stream_pool = 1;
     c.device = s->device;
@@ -381,16 +382,16 @@ bool launch_batch(od_server *s, std::vector<KArgs> &hk, std::vector<int32_t> &hf
         cudaError_t e;
         if (s->batch_steps > 1) {
             int bps = 0;
-            e = od::persistent_multi_occupancy(shapes[g][0], shapes[g][1], s->arith, smem, OD_STENCIL_3D7, &bps);
+            e = od::persistent_multi_occupancy(shapes[g][0], shapes[g][1], od::kernel_mode(s->arith, true), smem, OD_STENCIL_3D7, &bps);
             int32_t *q = s->d_queue + slot * kShapes + g;
             if (e == cudaSuccess && bps < 1) e = cudaErrorInvalidConfiguration;
             if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, sizeof(int32_t), s->compute);
             if (e == cudaSuccess)
                 e = od::launch_persistent_multi(dj, df, nj, steps, q, geom,
                                                 std::min(grid[(size_t)g], bps * s->num_sms), shapes[g][0],
-                                                shapes[g][1], s->arith, smem, OD_STENCIL_3D7, s->compute);
+                                                shapes[g][1], od::kernel_mode(s->arith, true), smem, OD_STENCIL_3D7, s->compute);
         } else {
-            e = od::launch_tiles_multi(dj, df, nj, geom, grid[(size_t)g], shapes[g][0], shapes[g][1], s->arith, smem,
+            e = od::launch_tiles_multi(dj, df, nj, geom, grid[(size_t)g], shapes[g][0], shapes[g][1], od::kernel_mode(s->arith, true), smem,
                                        OD_STENCIL_3D7, s->compute);
         }
         if (e != cudaSuccess) {
@@ -586,7 +587,7 @@ od_status od_server_create(od_server **out, const od_server_config *cfg) {
     s->threads = auto_shape ? 0 : cfg->threads ? cfg->threads : 128;
     s->cpt = auto_shape ? 0 : cfg->cells_per_thread ? cfg->cells_per_thread : 4;
     s->stages = cfg->stages ? cfg->stages : 4;
-    s->arith = cfg->arith >= 0 ? cfg->arith : 12;
+    s->arith = cfg->arith >= 0 ? cfg->arith : od::kDefaultArith;
     s->max_jobs = cfg->max_jobs_per_launch > 0 ? cfg->max_jobs_per_launch : 256;
     s->batch_steps = cfg->batch_steps > 0 ? cfg->batch_steps : 8;
     if (cfg->batch_steps < 0 || cfg->batch_steps > 4096) {
@@ -652,7 +653,7 @@ od_status od_server_create(od_server **out, const od_server_config *cfg) {
     for (int g = 0; g < kShapes; ++g) {
         if (s->threads && g > 0) break;  // one fixed shape
         const int nt = s->threads ? s->threads : kAutoShapes[g][0], ct = s->threads ? s->cpt : kAutoShapes[g][1];
-        if (od::prepare_tile_kernels(nt, ct, s->arith, s->smem_cap, OD_STENCIL_3D7) != cudaSuccess)
+        if (od::prepare_tile_kernels(nt, ct, od::kernel_mode(s->arith, true), s->smem_cap, OD_STENCIL_3D7) != cudaSuccess)
             return bail(OD_ECUDA, "cannot configure the tile kernels");
     }
     s->worker = std::thread(worker_main, s);

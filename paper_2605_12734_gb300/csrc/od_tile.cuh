@@ -139,6 +139,16 @@ static __device__ __noinline__ double update_slow(double W, double E, double S, 
     return jacobi_update_ieee<true>(W, E, S, N, D, U);
 }
 
+// The same for a field of fixed-point words (base exponent e0); the cell is
+// given by its address in the planes below, of and above it.
+static __device__ __noinline__ double update_slow_fx(const double *sd, const double *sc, const double *su, int pitch,
+                                                     uint32_t e0) {
+    const double v = jacobi_update_ieee<true>(fx_decode(f64_bits(sc[-1]), e0), fx_decode(f64_bits(sc[1]), e0),
+                                              fx_decode(f64_bits(sc[-pitch]), e0), fx_decode(f64_bits(sc[pitch]), e0),
+                                              fx_decode(f64_bits(*sd), e0), fx_decode(f64_bits(*su), e0));
+    return f64_from(fx_encode(v, e0));
+}
+
 // Which thread refills a ring slot: lane 0 of a different warp each plane
 // (1) or thread 0 always (0); a build may choose (-DOD_ROTATE_ISSUE=0).
 #ifndef OD_ROTATE_ISSUE
@@ -151,9 +161,14 @@ struct Ring {
     uint32_t seq;      // planes issued by this CTA before the current tile
 };
 
-// The anchored arithmetic's parameters for one launch: the window anchor for
-// cells with one or no FP64 add (e0), +1 for cells with two or three, and
-// the run-time 1 of the multiply-adds.
+// Arithmetic mode of a sweep over fixed-point field words (od_arith.cuh):
+// what the default mode 12 runs on a context that holds its field that way.
+constexpr int kFx = 16;
+
+// The arithmetic's parameters for one launch: the window anchor for cells
+// with one or no FP64 add (e0), +1 for cells with two or three, and the
+// run-time 1 of the multiply-adds; or the base exponent (e0) of a field of
+// fixed-point words.
 struct Arith {
     uint32_t e0, one;
 };
@@ -162,6 +177,10 @@ template <int AM>
 __device__ __forceinline__ Arith arith_setup(const KArgs &a, const KArgs &g) {
     Arith r;
     r.one = g.one;  // from the kernel parameter g (a constant-bank operand, no register)
+    if constexpr (AM == kFx) {
+        r.e0 = a.fmt->base;
+        return r;
+    }
     r.e0 = AM >= 12 ? anchor_for(a.vmax ? *a.vmax : 0ull, 1) : 0u;
     return r;
 }
@@ -193,7 +212,9 @@ template <int AM>
 __device__ __forceinline__ double update_cell(const double *sd, const double *sc, const double *su, int r, int pitch,
                                               int m, const Arith &ar, bool &ok) {
     const double W = sc[r - 1], E = sc[r + 1], S = sc[r - pitch], N = sc[r + pitch], D = sd[r], U = su[r];
-    if constexpr (AM == 12) {
+    if constexpr (AM == kFx) {
+        return f64_from(fx_update3(f64_bits(W), f64_bits(E), f64_bits(S), f64_bits(N), f64_bits(D), f64_bits(U), ok));
+    } else if constexpr (AM == 12) {
         return jacobi_update_anchored<2>(W, E, S, N, D, U, ar.e0 + 1u, ok, ar.one);
     } else if constexpr (AM == 13) {
         return jacobi_update_anchored<1>(W, E, S, N, D, U, ar.e0, ok, ar.one);
@@ -406,7 +427,9 @@ __device__ __forceinline__ bool run_tile(const KArgs &a, int tile_id, int sp, Ri
             const double *sc = ring.base + (size_t)sl_0 * SD;
             double *su = ring.base + (size_t)sl_p1 * SD;
             double *dpl = dst + (size_t)(k + 1) * plane;
-            uint32_t bad = 0;  // bit m: cell m left the integer routines' domain
+            // bit m: cell m left the integer routines' domain (a context that could
+            // not keep its field as words, base exponent 0, recomputes every cell)
+            uint32_t bad = AM == kFx && ar.e0 == 0u ? (1u << CPT) - 1u : 0u;
 #pragma unroll
             for (int m = 0; m < CPT; ++m) {
                 const int r = rf[m];
@@ -419,8 +442,12 @@ __device__ __forceinline__ bool run_tile(const KArgs &a, int tile_id, int sp, Ri
 #pragma unroll
                 for (int m = 0; m < CPT; ++m) {
                     const int r = rf[m];
-                    if (bad & (1u << m))
-                        dpl[r] = update_slow(sc[r - 1], sc[r + 1], sc[r - pitch], sc[r + pitch], sd[r], su[r]);
+                    if (bad & (1u << m)) {
+                        if constexpr (AM == kFx)
+                            dpl[r] = update_slow_fx(sd + r, sc + r, su + r, pitch, ar.e0);
+                        else
+                            dpl[r] = update_slow(sc[r - 1], sc[r + 1], sc[r - pitch], sc[r + pitch], sd[r], su[r]);
+                    }
                 }
             }
             if (patch_next) {  // plane k+1's x halo (its slot is only read at interior cells above)
@@ -462,6 +489,13 @@ static __device__ __noinline__ double update2d_slow(double W, double E, double S
     return jacobi2d_update_ieee<true>(W, E, S, N);  // the division by 4 as an exponent step where exact
 }
 
+static __device__ __noinline__ double update2d_slow_fx(const double *sd, const double *sc, const double *su,
+                                                       uint32_t e0) {
+    const double v = jacobi2d_update_ieee<true>(fx_decode(f64_bits(sc[-1]), e0), fx_decode(f64_bits(sc[1]), e0),
+                                                fx_decode(f64_bits(*sd), e0), fx_decode(f64_bits(*su), e0));
+    return f64_from(fx_encode(v, e0));
+}
+
 // The 2D 5-point sweep (the paper's Jacobi2D, Sec. V) on the internal grid
 // (nx, 1, ny): a chare's 2D rows are its planes, one row each, so A is the
 // padded 2D block and plane k (interior row k) starts at (k+1)*pitch.  A tile
@@ -476,7 +510,9 @@ static __device__ __noinline__ double update2d_slow(double W, double E, double S
 template <int AM>
 __device__ __forceinline__ double update_cell_2d(double W, double E, double S, double N, int m, const Arith &ar,
                                                  bool &ok) {
-    if constexpr (AM == 12) {
+    if constexpr (AM == kFx) {
+        return f64_from(fx_update2(f64_bits(W), f64_bits(E), f64_bits(S), f64_bits(N), ok));
+    } else if constexpr (AM == 12) {
         return jacobi2d_update_anchored<1>(W, E, S, N, ar.e0, ok, ar.one);
     } else if constexpr (AM == 13) {
         return jacobi2d_update_anchored<0>(W, E, S, N, ar.e0, ok, ar.one);
@@ -598,7 +634,9 @@ __device__ __forceinline__ bool run_tile_2d(const KArgs &a, int tile_id, int sp,
             double *dpl = dst + (size_t)(k + 1) * plane;
             // no validity branch: a slot past the segment's end repeats its
             // cell 0, so it stores the same value to the same place
-            uint32_t bad = 0;  // bit m: cell m left the integer routines' domain
+            // bit m: cell m left the integer routines' domain (a context that could
+            // not keep its field as words, base exponent 0, recomputes every cell)
+            uint32_t bad = AM == kFx && ar.e0 == 0u ? (1u << CPT) - 1u : 0u;
 #pragma unroll
             for (int m = 0; m < CPT; ++m) {
                 const int r = rf[m];
@@ -610,7 +648,12 @@ __device__ __forceinline__ bool run_tile_2d(const KArgs &a, int tile_id, int sp,
 #pragma unroll
                 for (int m = 0; m < CPT; ++m) {
                     const int r = rf[m];
-                    if (bad & (1u << m)) dpl[r] = update2d_slow(sc[r - 1], sc[r + 1], sd[r], su[r]);
+                    if (bad & (1u << m)) {
+                        if constexpr (AM == kFx)
+                            dpl[r] = update2d_slow_fx(sd + r, sc + r, su + r, ar.e0);
+                        else
+                            dpl[r] = update2d_slow(sc[r - 1], sc[r + 1], sd[r], su[r]);
+                    }
                 }
             }
             if (xg) su[patch_dst] = xv;  // row k+1's x halo (its slot is only read at the cells above)

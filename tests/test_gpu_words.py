@@ -1,0 +1,135 @@
+"""The sweep over fixed-point field words on the GPU where its formats and its
+schedule have edges, bit for bit against the CPU oracle: fields that leave,
+straddle or outgrow the window, an import that changes the format of a running
+context, faces fed from outside, and tiles with long dependency lists, one
+plane, one row or deep rings."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+PATHS = ["persistent", "fused", "fused_graph", "per_chare", "graph"]
+
+
+@pytest.fixture(scope="module")
+def od():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2605_12734_gb300 import build
+    build.build()
+    import paper_2605_12734_gb300 as pkg
+    return pkg
+
+
+def same(got, want):
+    return np.array_equal(np.ascontiguousarray(got).view(np.uint64), np.ascontiguousarray(want).view(np.uint64))
+
+
+def field(kind, n, rng):
+    u = rng.random(n)
+    if kind == "edges":  # the window's ends, one step inside and outside of them, and powers of two
+        ends = [1.0, np.nextafter(1.0, 0), np.nextafter(1.0, 2), 2.0 ** -8, np.nextafter(2.0 ** -8, 0),
+                np.nextafter(2.0 ** -8, 1), 0.5, 0.25, 2.0 ** -7]
+        return rng.choice(ends, n)
+    if kind == "tiny":   # window values among ones far below it, zeros of both signs and subnormals
+        v = np.where(u < 0.5, u, np.exp2(-rng.integers(9, 1070, n).astype(np.float64)))
+        v[::5] = 0.0
+        v[1::17] = -0.0
+        v[2::23] = 5e-324
+        return v
+    if kind == "huge":   # near the top of the double range, some sums overflow
+        return u * 1.5e308
+    if kind == "infinite":
+        u[::97] = np.inf
+        return u
+    return u
+
+
+def solve_from(nx, ny, nz, seed, interior, iters):
+    if nz == 0:
+        P = oracle.init_padded_2d(nx, ny, seed, 1)
+        P[1:-1, 1:-1] = interior.reshape(ny, nx)
+        return oracle.sweep_2d(P, iters)[1:-1, 1:-1].ravel()
+    P = oracle.init_padded(nx, ny, nz, seed, 1)
+    P[1:-1, 1:-1, 1:-1] = interior.reshape(nz, ny, nx)
+    return oracle.interior(oracle.sweep(P, iters))
+
+
+@pytest.mark.parametrize("path", PATHS)
+@pytest.mark.parametrize("kind", ["edges", "tiny", "huge", "infinite"])
+def test_fields_outside_the_window(od, path, kind):
+    nx, ny, nz, seed, iters = 37, 30, 26, 5, 6
+    u = field(kind, nx * ny * nz, np.random.default_rng(len(kind)))
+    want = solve_from(nx, ny, nz, seed, u, iters)
+    with od.Jacobi3D(nx, ny, nz, split=(2, 3, 2), seed=seed, path=path) as s:
+        s.write(u)
+        s.step(iters)
+        assert same(s.read(), want)
+        probe = np.array([0, 1, nx, nx * ny - 1, nx * ny * nz - 1, 4321])
+        assert same(s.read_cells(probe), want[probe])
+
+
+@pytest.mark.parametrize("path", PATHS)
+def test_import_that_changes_the_format(od, path):
+    # each field's largest value asks for another window than the one before,
+    # the last for none; the Dirichlet shell and the ghost layers follow
+    nx, ny, nz, seed = 45, 21, 33, 9
+    rng = np.random.default_rng(3)
+    with od.Jacobi3D(nx, ny, nz, split=(3, 2, 2), seed=seed, path=path) as s:
+        for scale in (1.0, 3e4, 1e200, 1.0, 1e280):
+            u = rng.random(nx * ny * nz) * scale
+            s.write(u)
+            s.step(3)
+            assert same(s.read(), solve_from(nx, ny, nz, seed, u, 3)), scale
+
+
+@pytest.mark.parametrize("path", ["persistent", "per_chare", "fused_graph"])
+def test_faces_fed_from_outside(od, path):
+    # an imported face may hold anything: the context leaves its words
+    nx, ny, nz, seed, iters = 28, 22, 19, 4, 5
+    rng = np.random.default_rng(8)
+    P = oracle.init_padded(nx, ny, nz, seed, 1)
+    mid = oracle.sweep(P, 2)
+    face = rng.random(nz * ny) * 1e290
+    mid[1:-1, 1:-1, 0] = face.reshape(nz, ny)
+    want = oracle.interior(oracle.sweep(mid, iters))
+    with od.Jacobi3D(nx, ny, nz, split=(2, 2, 2), seed=seed, path=path) as s:
+        s.step(2)
+        s.face_copy(0, 1, face)  # the ghost layer of the parity that the next step reads
+        s.step(1)
+        s.face_copy(0, 1, face)  # and of the other one
+        s.step(iters - 1)
+        assert same(s.read(), want)
+        out = np.empty(nz * ny)
+        s.face_copy(1, 0, out)
+        assert same(out, want.reshape(nz, ny, nx)[:, :, nx - 1].ravel())
+
+
+@pytest.mark.parametrize("kw", [
+    dict(cuts=([0, 4, 260], [0, 128], [0, 3])),                       # a tile that reads more than 20 others
+    dict(cuts=([0, 1, 2, 260], [0, 1, 128], [0, 1, 3]), tile_z=1),     # single cells, rows and planes
+    dict(split=(2, 2, 1), stages=3, tile_z=2), dict(split=(2, 2, 1), stages=8, tile_z=1),
+    dict(split=(3, 2, 3), threads=512, cells_per_thread=1), dict(split=(1, 4, 1), threads=256, cells_per_thread=8),
+])
+@pytest.mark.parametrize("path", ["persistent", "fused"])
+def test_tile_shapes(od, path, kw):
+    want = oracle.solve(260, 128, 3, 6, 1, 7)
+    with od.Jacobi3D(260, 128, 3, seed=6, path=path, **kw) as s:
+        s.step(3)
+        s.step(4)
+        assert same(s.read(), want)
+
+
+@pytest.mark.parametrize("kind", ["edges", "tiny", "huge", "infinite"])
+@pytest.mark.parametrize("path", ["persistent", "fused", "per_chare"])
+def test_2d_fields_outside_the_window(od, path, kind):
+    nx, ny, seed, iters = 143, 61, 5, 7
+    u = field(kind, nx * ny, np.random.default_rng(len(kind)))
+    want = solve_from(nx, ny, 0, seed, u, iters)
+    with od.Jacobi2D(nx, ny, split=(3, 2), seed=seed, path=path) as s:
+        s.write(u)
+        s.step(iters)
+        assert same(s.read(), want)
