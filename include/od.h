@@ -134,7 +134,9 @@ typedef struct od_config {
                                     device memory while tuning (skipped if
                                     that is not available). */
     int32_t tile_y;              /* max rows per tile (0 = planner default) */
-    int32_t tile_z;              /* planes per tile (0 = planner default) */
+    int32_t tile_z;              /* planes per tile (0 = 32; a context in the
+                                    default arithmetic runs fewer where that
+                                    leaves few tiles, 64 rows in 2D: od_stats) */
     int32_t threads;             /* threads per CTA: 128, 256 or 512 */
     int32_t cells_per_thread;    /* 1, 2, 4 or 8; supported pairs 128 x {2,4,8},
                                     256 x {1,2,4,8}, 512 x {1,2}.  Both 0: the

@@ -888,7 +888,7 @@ od_status create_context(od_ctx **out, const od_config *cfg_in, bool sync) {
     c->tune_ms = tune_ms;
     c->cfg.cuts_x = c->cfg.cuts_y = c->cfg.cuts_z = nullptr;  // not kept past the call
     std::string err;
-    od_status s = od::build_plan(cfg, &c->plan, &err);
+    od_status s = od::build_plan(cfg, &c->plan, &err, true, true);
     if (s != OD_OK) {
         release(c);
         return fail(s, err);

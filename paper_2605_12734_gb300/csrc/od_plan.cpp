@@ -59,30 +59,6 @@ bool edges_from(int64_t n, int32_t p, const int32_t *cuts, int32_t ncuts, const 
     return true;
 }
 
-struct Box {
-    int64_t lo[3], hi[3];
-};
-
-Box tile_box(const HostChare &c, const TileDev &t) {
-    Box b;
-    b.lo[0] = c.x0 + t.i0;    b.hi[0] = b.lo[0] + t.ni;
-    b.lo[1] = c.y0 + t.j0;    b.hi[1] = b.lo[1] + t.nj;
-    b.lo[2] = c.z0 + t.k0;    b.hi[2] = b.lo[2] + t.nk;
-    return b;
-}
-
-// Tiles whose cells a 7-point update of `a` reads, or that read `a`'s cells:
-// the same tile, or boxes that touch along one axis and overlap on the other
-// two.
-bool adjacent_or_same(const Box &a, const Box &b) {
-    int overlap = 0, touch = 0;
-    for (int d = 0; d < 3; ++d) {
-        if (a.lo[d] < b.hi[d] && b.lo[d] < a.hi[d]) ++overlap;
-        else if (a.hi[d] == b.lo[d] || b.hi[d] == a.lo[d]) ++touch;
-    }
-    return overlap == 3 || (overlap == 2 && touch == 1);
-}
-
 // split n into parts of at most `cap`, balanced
 void balanced_parts(int32_t n, int32_t cap, std::vector<int32_t> *starts, std::vector<int32_t> *lens) {
     int32_t parts = (n + cap - 1) / cap;
@@ -103,9 +79,92 @@ int32_t stage_doubles_for(int32_t nj, int32_t pitch) {
     return round_up((nj + 2) * pitch, 16);     // keep slots 128-byte aligned
 }
 
+// Tiles and dependency-list entries of the grid with tz planes per tile (the
+// shape, the tile rows and the cuts of p), as build_plan lays them out.
+static void count_tiles(const Plan &p, int32_t tz, int64_t *ntiles, int64_t *ndeps) {
+    const bool d3 = p.stencil == OD_STENCIL_3D7;
+    int64_t cap = (int64_t)p.threads * p.cpt;
+    if (!d3 && p.tile_y > 0) cap = std::min<int64_t>(cap, p.tile_y);
+    auto parts = [](int64_t n, int64_t most) { return (n + std::min(n, most) - 1) / std::min(n, most); };
+    const size_t nx = p.ex.size() - 1, ny = p.ey.size() - 1, nz = p.ez.size() - 1;
+    int64_t chunks = 0;  // over all block layers
+    for (size_t c = 0; c < nz; ++c) chunks += parts(p.ez[c + 1] - p.ez[c], tz);
+    auto rows = [&](size_t a) {  // rows of a tile in block column a
+        int64_t nj = std::max<int64_t>(1, cap / (p.ex[a + 1] - p.ex[a]));
+        return p.tile_y > 0 ? std::min<int64_t>(nj, p.tile_y) : nj;
+    };
+    int64_t slabs = 0, inside = 0, across = 0;  // tiles of a plane; pairs of them within a block, between blocks
+    for (size_t b = 0; b < ny; ++b) {
+        const int64_t by = p.ey[b + 1] - p.ey[b];
+        for (size_t a = 0; a < nx; ++a) {
+            int64_t n;
+            if (d3) {
+                n = parts(by, rows(a));
+            } else {  // segments of even width
+                const int64_t bx = p.ex[a + 1] - p.ex[a], w = (parts(bx, cap) + bx - 1) / parts(bx, cap);
+                n = parts(bx, w + (w & 1));
+            }
+            slabs += n;
+            inside += n - 1;
+            if (d3 && b + 1 < ny) across += 1;
+            if (a + 1 == nx) continue;
+            if (!d3) {
+                across += 1;
+                continue;
+            }
+            // slabs of the next column that share rows: both are balanced
+            // splits of the same rows, so each boundary that only one of them
+            // has adds one pair to the n of them
+            const int64_t m = parts(by, rows(a + 1));
+            int64_t i = 0, j = 0, pairs = 0;
+            auto end = [&](int64_t k, int64_t of) { return (k + 1) * (by / of) + std::min(k + 1, by % of); };
+            while (i < n && j < m) {
+                ++pairs;
+                const int64_t ei = end(i, n), ej = end(j, m);
+                if (ei <= ej) ++i;
+                if (ej <= ei) ++j;
+            }
+            across += pairs;
+        }
+    }
+    *ntiles = slabs * chunks;
+    // itself, both ways: within a plane, and from each plane chunk to the next
+    *ndeps = slabs * chunks + 2 * (inside + across) * chunks + 2 * slabs * (chunks - 1);
+}
+
+// Bytes of the per-tile tables in the arena.
+static size_t table_bytes(int64_t nt, int64_t nd) {
+    auto a = [](size_t v) { return align_up(v, kAlign); };
+    return a((size_t)nt * 4) + a((size_t)nt * sizeof(TileDev)) + a(((size_t)nt + 1) * 4) +
+           a((size_t)std::max<int64_t>(1, nd) * 4) + a((size_t)nt * 4) + a((size_t)nt * sizeof(TileRec));
+}
+
+// Planes (2D: rows) per tile that a context's sweep over words runs with when
+// none is asked for.  Tall tiles copy fewer halo planes, but a grid of few
+// tiles leaves CTAs idle and makes every step wait for its slowest tile; about
+// two tiles per resident CTA keep the CTAs busy across steps.  So: the tallest
+// that gives 1800 tiles, 4 where none does, 2 where that leaves fewer than
+// 800.  Measured, us a step with 32 planes and with the rule's: 64^3 in 8
+// chares 24.6 / 8.0, 100^3 in 8 21.0 / 11.4, 128^3 in 64 26.5 / 13.6, 203^3 in
+// 27 45.6 / 35.4, 256^3 in 64 72.4 / 60.8; 300^3 in 216 98.2 with 32 (2160
+// tiles), 101.6 with 16.  2D: 96 x 64 in 4 20.0 / 4.9, 1000 x 777 in 16 18.1 /
+// 8.4, 2048^2 in 16 26.0 / 13.4, 5000 x 3000 in 16 49.7 / 44.0, 8192^2 in 256
+// 169 / 165 (64 rows), 16384^2 in 1024 678 / 662.
+static int32_t words_tile_z(const Plan &p) {
+    const bool d3 = p.stencil == OD_STENCIL_3D7;
+    auto tiles_with = [&](int32_t tz) {
+        int64_t nt = 0, nd = 0;
+        count_tiles(p, tz, &nt, &nd);
+        return nt;
+    };
+    int32_t tz = d3 ? 32 : 64;
+    while (tz > 4 && tiles_with(tz) < 1800) tz /= 2;
+    return tz == 4 && tiles_with(4) < 800 ? 2 : tz;
+}
+
 od_status build_plan(const od_config *cfg, Plan *P, std::string *err) { return build_plan(cfg, P, err, true); }
 
-od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_gpu) {
+od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_gpu, bool running) {
     Plan &p = *P;
     p = Plan();
     if (!cfg) { *err = "null config"; return OD_EINVAL; }
@@ -322,6 +381,10 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     p.bytes_per_step = 16.0 * (double)p.cells + 16.0 * (double)p.face_internal +
                        8.0 * (double)p.face_dirichlet;
 
+    // a context runs the default arithmetic with its own planes per tile
+    const int32_t run_z = cfg->tile_z == 0 && p.amode == kDefaultArith ? words_tile_z(p) : 0;
+    const int32_t tile_z = cfg->tile_z > 0 ? cfg->tile_z : running && run_z ? run_z : 32;
+
     // tiles: full rows, balanced row slabs and plane chunks
     std::vector<int32_t> js, jl, ks, kl;
     int32_t max_stage = 0;
@@ -333,8 +396,7 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
         if (p.tile_y > 0) cap = std::min(cap, p.tile_y);  // tile_y caps the segment for 2D
         const int32_t nseg = (h.bx + cap - 1) / cap;
         const int32_t w = round_up((h.bx + nseg - 1) / nseg, 2);
-        int32_t tz = p.tile_z > 0 ? p.tile_z : 32;
-        tz = std::min(tz, h.bz);
+        const int32_t tz = std::min(tile_z, h.bz);
         balanced_parts(h.bz, tz, &ks, &kl);
         h.tile_begin = (int32_t)p.tiles.size();
         h.ti.clear();
@@ -365,8 +427,7 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
         int32_t nj_cap = (p.threads * p.cpt) / h.bx;
         if (p.tile_y > 0) nj_cap = std::min(nj_cap, p.tile_y);
         nj_cap = std::max(1, std::min(nj_cap, h.by));
-        int32_t tz = p.tile_z > 0 ? p.tile_z : 32;
-        tz = std::min(tz, h.bz);
+        const int32_t tz = std::min(tile_z, h.bz);
         balanced_parts(h.by, nj_cap, &js, &jl);
         balanced_parts(h.bz, tz, &ks, &kl);
         h.tile_begin = (int32_t)p.tiles.size();
@@ -423,38 +484,55 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     }
     p.smem_bytes = (int32_t)smem;
 
-    // dependency lists (tiles of the chare itself and its six neighbours):
-    // per axis only the candidate's tiles within one cell of the tile's range
-    // can touch it, found by bisection over the chare's tile starts
+    // Dependency lists: the tiles of the chare itself and its six neighbours
+    // whose boxes touch the tile's on a face.  A neighbour shares the extents
+    // of the other two axes, so their partitions too, except that the rows per
+    // tile follow the row length: across an x face the slabs are matched by
+    // their rows.
     p.dep_ptr.assign(p.tiles.size() + 1, 0);
     p.dep_idx.clear();
-    for (size_t ti = 0; ti < p.tiles.size(); ++ti) {
-        const TileDev &t = p.tiles[ti];
-        const HostChare &h = p.ch[(size_t)t.c];
-        Box a = tile_box(h, t);
-        int32_t cand[7] = {t.c, h.nbr[0], h.nbr[1], h.nbr[2], h.nbr[3], h.nbr[4], h.nbr[5]};
-        for (int q = 0; q < 7; ++q) {
-            if (cand[q] < 0) continue;
-            const HostChare &g = p.ch[(size_t)cand[q]];
-            const std::vector<int32_t> *st[3] = {&g.ti, &g.tj, &g.tk};
-            const int64_t org[3] = {g.x0, g.y0, g.z0};
-            size_t lo[3], hi[3];
-            for (int d = 0; d < 3; ++d) {
-                // tiles whose start is <= a.hi (chare-local), from the last one starting <= a.lo - 1
-                const std::vector<int32_t> &v = *st[d];
-                const int64_t l = a.lo[d] - 1 - org[d], r = a.hi[d] - org[d];
-                size_t first = (size_t)(std::upper_bound(v.begin(), v.end(), l) - v.begin());
-                lo[d] = first > 0 ? first - 1 : 0;
-                hi[d] = (size_t)(std::upper_bound(v.begin(), v.end(), r) - v.begin());
-            }
-            for (size_t e = lo[2]; e < hi[2]; ++e)
-                for (size_t b = lo[1]; b < hi[1]; ++b)
-                    for (size_t i = lo[0]; i < hi[0]; ++i) {
-                        const int32_t u = g.tile_begin + (int32_t)((e * g.tj.size() + b) * g.ti.size() + i);
-                        if (adjacent_or_same(a, tile_box(g, p.tiles[(size_t)u]))) p.dep_idx.push_back(u);
+    p.dep_idx.reserve(8 * p.tiles.size());
+    for (size_t c = 0; c < p.ch.size(); ++c) {
+        const HostChare &h = p.ch[c];
+        const int32_t ni = (int32_t)h.ti.size(), nb = (int32_t)h.tj.size(), ne = (int32_t)h.tk.size();
+        const HostChare *nbr[6];
+        for (int f = 0; f < 6; ++f) nbr[f] = h.nbr[f] >= 0 ? &p.ch[(size_t)h.nbr[f]] : nullptr;
+        int32_t t = h.tile_begin;
+        for (int32_t e = 0; e < ne; ++e)
+            for (int32_t b = 0; b < nb; ++b) {
+                const int32_t j0 = h.tj[b], j1 = b + 1 < nb ? h.tj[b + 1] : h.by;
+                for (int32_t i = 0; i < ni; ++i, ++t) {
+                    std::vector<int32_t> &d = p.dep_idx;
+                    if (e > 0) d.push_back(t - ni * nb);
+                    if (b > 0) d.push_back(t - ni);
+                    if (i > 0) d.push_back(t - 1);
+                    d.push_back(t);
+                    if (i + 1 < ni) d.push_back(t + 1);
+                    if (b + 1 < nb) d.push_back(t + ni);
+                    if (e + 1 < ne) d.push_back(t + ni * nb);
+                    for (int side = 0; side < 2; ++side) {  // x faces
+                        const HostChare *g = nbr[OD_FACE_XLO + side];
+                        if (!g || i != (side ? ni - 1 : 0)) continue;
+                        const int32_t gi = (int32_t)g->ti.size(), gb = (int32_t)g->tj.size();
+                        int32_t q = (int32_t)(std::upper_bound(g->tj.begin(), g->tj.end(), j0) - g->tj.begin()) - 1;
+                        for (; q < gb && g->tj[q] < j1; ++q)
+                            d.push_back(g->tile_begin + (e * gb + q) * gi + (side ? 0 : gi - 1));
                     }
-        }
-        p.dep_ptr[ti + 1] = (int32_t)p.dep_idx.size();
+                    for (int side = 0; side < 2; ++side) {  // y faces
+                        const HostChare *g = nbr[OD_FACE_YLO + side];
+                        if (!g || b != (side ? nb - 1 : 0)) continue;
+                        const int32_t gb = (int32_t)g->tj.size();
+                        d.push_back(g->tile_begin + (e * gb + (side ? 0 : gb - 1)) * ni + i);
+                    }
+                    for (int side = 0; side < 2; ++side) {  // z faces
+                        const HostChare *g = nbr[OD_FACE_ZLO + side];
+                        if (!g || e != (side ? ne - 1 : 0)) continue;
+                        const int32_t ge = (int32_t)g->tk.size();
+                        d.push_back(g->tile_begin + ((side ? 0 : ge - 1) * nb + b) * ni + i);
+                    }
+                    p.dep_ptr[(size_t)t + 1] = (int32_t)d.size();
+                }
+            }
     }
     p.order.resize(p.tiles.size());
     for (size_t ti = 0; ti < p.tiles.size(); ++ti) p.order[ti] = (int32_t)ti;
@@ -506,6 +584,13 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
         h.offRecv[1] = take(f_bytes);
     }
     p.arena_bytes = at;
+    if (!running && run_z && run_z != tile_z) {
+        // the arena also holds the tables of the tiles a context will run with
+        int64_t nt = 0, nd = 0;
+        count_tiles(p, run_z, &nt, &nd);
+        const size_t mine = table_bytes((int64_t)p.tiles.size(), (int64_t)p.dep_idx.size()), run = table_bytes(nt, nd);
+        if (run > mine) p.arena_bytes += run - mine;
+    }
     return OD_OK;
 }
 
