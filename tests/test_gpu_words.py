@@ -133,3 +133,25 @@ def test_2d_fields_outside_the_window(od, path, kind):
         s.write(u)
         s.step(iters)
         assert same(s.read(), want)
+
+
+# below a million cells the entry sweeps doubles, above words; rows and planes
+# that do not divide a block, one plane, one row and columns of one cell
+@pytest.mark.parametrize("dims", [(7, 300, 5), (131, 127, 65), (1100, 1000, 1), (3, 1, 400000), (1, 5003, 211)])
+@pytest.mark.parametrize("kind", ["uniform", "edges", "tiny", "huge"])
+def test_allocation_free_entry(od, dims, kind):
+    import torch
+    nx, ny, nz = dims
+    rng = np.random.default_rng(nx)
+    P = field(kind, (nx + 2) * (ny + 2) * (nz + 2), rng).reshape(nz + 2, ny + 2, nx + 2)
+    for iters in (3, 7, 8):
+        want = oracle.sweep(P.copy(), iters)
+        u = torch.from_numpy(P.ravel().copy()).to("cuda:0")
+        out = torch.full_like(u, -1.0)
+        od.jacobi_noalloc(u, out, nx, ny, nz, iters)
+        torch.cuda.synchronize()
+        got = out.cpu().numpy().reshape(P.shape)
+        assert same(got[1:-1, 1:-1, 1:-1], want[1:-1, 1:-1, 1:-1]), iters
+        shell = np.ones(P.shape, dtype=bool)
+        shell[1:-1, 1:-1, 1:-1] = False
+        assert same(got[shell], P[shell])  # carried over unchanged
