@@ -120,15 +120,15 @@ od_status enqueue_persistent(od_ctx *c, int32_t iters) {
     int32_t done = 0;
     while (done < iters) {
         int32_t n = std::min(iters - done, chunk_max);
-        OD_CUDA(cudaMemsetAsync(c->d_queue, 0, sizeof(int32_t), c->stream));
-        OD_CUDA(cudaMemsetAsync(c->d_epoch, 0, (size_t)nt * sizeof(int32_t), c->stream));
+        // the ticket counter lies right before the step counters: one memset
+        OD_CUDA(cudaMemsetAsync(c->d_queue, 0, (size_t)(nt + 1) * sizeof(int32_t), c->stream));
         KArgs a = base_args_impl(c);
         a.iters = n;
         a.t0 = (int32_t)(c->steps & 0x7fffffff);
         OD_CUDA(od::launch_persistent(a, grid, p.threads, p.cpt, c->kernel_mode(), p.smem_bytes, c->stream));
         c->steps += n;
         c->launches++;
-        c->api_calls += 3;
+        c->api_calls += 2;
         done += n;
     }
     return OD_OK;
@@ -415,8 +415,13 @@ od_status enqueue_fused_graph(od_ctx *c, int32_t iters) {
     return s;
 }
 
+// Wait for the context's stream and read its error record.  The record's copy
+// is queued behind the work and lands in pageable memory, so one blocking call
+// does both (a stream wait and a blocking copy after it took 10 us more).
 od_status check_device_error_impl(od_ctx *c) {
-    cudaError_t e = cudaStreamSynchronize(c->stream);
+    ErrDev h;
+    cudaError_t e = cudaMemcpyAsync(&h, c->d_err, sizeof h, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess && c->copy_pending) {
         e = cudaStreamSynchronize(c->copy_stream);
         c->copy_pending = false;
@@ -424,12 +429,6 @@ od_status check_device_error_impl(od_ctx *c) {
     if (e != cudaSuccess) {
         c->failed = true;
         return cuda_fail(e, "cudaStreamSynchronize");
-    }
-    ErrDev h;
-    e = cudaMemcpy(&h, c->d_err, sizeof h, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) {
-        c->failed = true;
-        return cuda_fail(e, "cudaMemcpy(error record)");
     }
     if (h.code != 0) {
         c->failed = true;
@@ -940,14 +939,14 @@ od_status create_context(od_ctx **out, const od_config *cfg_in, bool sync) {
     }
     char *A = c->arena;
     c->d_err = (ErrDev *)(A + p.off_err);
-    c->d_queue = (int32_t *)(A + p.off_queue);
     c->d_epoch = (int32_t *)(A + p.off_epoch);
+    c->d_queue = c->d_epoch - 1;  // the last word of the queue block's alignment
     c->d_ch = (ChareDev *)(A + p.off_chares);
     c->d_tiles = (TileDev *)(A + p.off_tiles);
     c->d_dep_ptr = (int32_t *)(A + p.off_dep_ptr);
     c->d_dep_idx = (int32_t *)(A + p.off_dep_idx);
     c->d_order = (int32_t *)(A + p.off_order);
-    c->d_vmax = (uint64_t *)(A + p.off_queue + 8);  // the queue block holds 64 bytes
+    c->d_vmax = (uint64_t *)(A + p.off_queue + 8);  // the queue block holds 256 bytes
     c->d_fmt = (FmtDev *)(A + p.off_queue + 16);
     c->words = p.amode == od::kDefaultArith;
     c->h_ch.resize(p.ch.size());
@@ -1117,23 +1116,26 @@ od_status od_read_cells(od_ctx *c, const int64_t *cells, int64_t n, double *out)
 od_status od_read(od_ctx *c, double *dst, int32_t dst_is_device) {
     if (!c || !dst) return fail(OD_EINVAL, "null argument");
     DeviceGuard dg(c->device);
-    od_status s = check_device_error_impl(c);
-    if (s != OD_OK) return s;
     const od::Plan &p = c->plan;
     const int par = (int)(c->steps & 1);
     double *mapped = dst_is_device ? nullptr : device_view(dst);
+    od_status s = OD_OK;
+    cudaError_t e = cudaSuccess;
+    // the export follows the steps on the stream, and one wait at the end
+    // covers both and the error record
     if (dst_is_device || mapped) {
-        OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, dst_is_device ? dst : mapped,
-                                  c->d_fmt, c->stream));
+        e = od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, dst_is_device ? dst : mapped, c->d_fmt,
+                              c->stream);
     } else {
         s = ensure_stage(c);
         if (s != OD_OK) return s;
-        OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, c->d_stage, c->d_fmt, c->stream));
-        OD_CUDA(cudaMemcpyAsync(dst, c->d_stage, (size_t)p.cells * sizeof(double), cudaMemcpyDeviceToHost,
-                                c->stream));
+        e = od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, c->d_stage, c->d_fmt, c->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(dst, c->d_stage, (size_t)p.cells * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     }
-    OD_CUDA(cudaStreamSynchronize(c->stream));
-    return OD_OK;
+    s = check_device_error_impl(c);
+    if (s == OD_OK && e != cudaSuccess) s = cuda_fail(e, "od_read");
+    return s;
 }
 
 od_status od_write(od_ctx *c, const double *src, int32_t src_is_device) {

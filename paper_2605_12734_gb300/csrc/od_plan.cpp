@@ -567,7 +567,7 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
         return o;
     };
     p.off_err = take(sizeof(ErrDev));
-    p.off_queue = take(64);
+    p.off_queue = take(kAlign);  // largest value, format; its last word is the ticket counter
     p.off_epoch = take(p.tiles.size() * sizeof(int32_t));
     p.off_chares = take(p.ch.size() * sizeof(ChareDev));
     p.off_tiles = take(p.tiles.size() * sizeof(TileDev));
