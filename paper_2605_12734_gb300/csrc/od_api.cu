@@ -954,7 +954,7 @@ od_status create_context(od_ctx **out, const od_config *cfg_in, bool sync) {
         const od::HostChare &h = p.ch[i];
         ChareDev &d = c->h_ch[i];
         memset(&d, 0, sizeof d);
-        d.bx = h.bx; d.by = h.by; d.bz = h.bz; d.pitch = h.pitch;
+        d.bx = h.bx; d.by = h.by; d.bz = h.bz; d.pitch = h.pitch; d.col0 = h.col0;
         d.rows = h.rows; d.row0 = h.row0;
         for (int f = 0; f < 6; ++f) d.nbr[f] = h.nbr[f];
         for (int f = 0; f < 7; ++f) d.foff[f] = h.foff[f];
@@ -1095,7 +1095,7 @@ od_status od_read_cells(od_ctx *c, const int64_t *cells, int64_t n, double *out)
         const size_t ci = (size_t)cx + (size_t)p.px * ((size_t)cy + (size_t)p.py * (size_t)cz);
         const ChareDev &C = c->h_ch[ci];
         const int64_t i = x - C.x0, j = y - C.y0, k = z - C.z0;
-        addr[(size_t)q] = C.A[par] + ((k + 1) * C.rows + j + C.row0) * (int64_t)C.pitch + i + 1;
+        addr[(size_t)q] = C.A[par] + ((k + 1) * C.rows + j + C.row0) * (int64_t)C.pitch + C.col0 + i;
     }
     void *d_addr = nullptr, *d_out = nullptr;
     cudaError_t e = cudaMalloc(&d_addr, (size_t)n * sizeof(void *));

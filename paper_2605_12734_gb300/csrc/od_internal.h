@@ -2,12 +2,22 @@
 // of libod (overdecomposed 3D 7-point FP64 Jacobi on one GPU).
 //
 // Memory layout of one chare (block) in HBM, per parity p in {0,1}:
-//   A[p] : (bz+2) planes x (by+2) rows x pitch doubles, pitch = bx+2 rounded
-//          up to 2 (every row starts 16-byte aligned).  Plane 0 / bz+1 are the
-//          z-ghost planes, row 0 / by+1 of every plane the y-ghost rows,
-//          column 0 / bx+1 of every row the x-ghost cells, columns [1,bx] the
-//          cells; a last column may be padding.
-//          Interior cell (i,j,k) is A[p][((k+1)*(by+2) + (j+1))*pitch + i+1].
+//   A[p] : (bz+2) planes x (by+2) rows x pitch doubles.  Plane 0 / bz+1 are the
+//          z-ghost planes, row 0 / by+1 of every plane the y-ghost rows.  A
+//          row's cells are its columns [col0, col0+bx), its x-ghost cells the
+//          words before and after them.  Interior cell (i,j,k) is
+//          A[p][((k+1)*(by+2) + (j+1))*pitch + col0 + i].
+//          bx a multiple of 4: col0 = 4, pitch = bx+4, so cells fill whole
+//          32-byte sectors and the ghosts lie in sectors of their own (the x+
+//          ghost in the next row's column 0, and one word past the last row,
+//          for which the allocation has room).  A sweep stores only cells; L2
+//          then need not read a sector from HBM to complete it.  Measured with
+//          the ghosts adjacent and apart, 384^3 in 32^3 chares: 1.37 and 1.25
+//          bytes read for every byte of the field, 1.04 and 0.97 written;
+//          512^3 0.493 and 0.460 ms a step; 16384^2 0.678 and 0.646 ms.
+//          Otherwise col0 = 1, pitch = bx+2 rounded up to 2: ragged rows have
+//          partial sectors either way, and the shorter pitch copies less
+//          (41-cell rows 4 % faster than padded to 4).
 // A tile of full rows plus its two y-halo rows is then one contiguous run
 // that already holds the x-ghosts, fetched by a single 1D bulk copy (TMA),
 // and in shared memory x-1 / x+1 are the neighbouring words for every cell.
@@ -17,7 +27,7 @@
 // The 2D 5-point stencil runs on the internal grid (nx, 1, ny): a chare's 2D
 // rows are its "planes", and a plane is a single row (rows = 1, no y-ghost
 // rows), so A[p] is the chare's padded 2D block, (bz+2) rows x pitch:
-// interior cell (i, k) is A[p][(k+1)*pitch + i+1].  In general a plane holds
+// interior cell (i, k) is A[p][(k+1)*pitch + col0 + i].  In general a plane holds
 // `rows` rows and interior row j sits at row j + row0 of it: rows = by+2,
 // row0 = 1 in 3D; rows = 1, row0 = 0 in 2D.
 //
@@ -48,6 +58,7 @@
 struct ChareDev {
     int32_t bx, by, bz;     // interior extents
     int32_t pitch;          // row stride of A, doubles
+    int32_t col0;           // column of a row's first cell: 4 or 1
     int32_t rows, row0;     // rows per plane; row of interior row 0 in a plane
     int32_t nbr[6];         // neighbour per face or -1 (Dirichlet)
     int32_t foff[7];        // face offsets inside send/recv buffers (doubles)
@@ -80,12 +91,13 @@ struct alignas(256) TileRec {
     const double *zlo[2];    // the z neighbours' boundary plane, the tile's rows
     const double *zhi[2];
     int32_t bx, pitch, plane;           // row cells; doubles per row, per plane
+    int32_t cell0;           // ring-slot offset of a row's (2D: the segment's) first cell
     int32_t rows, cells;                // rows of the tile (1 in 2D), cells of a plane of it
     int32_t k0, nk, bz;                 // planes computed, planes of the chare
     int32_t xlo_pitch, xlo_plane, xhi_pitch, xhi_plane, ylo_plane, yhi_plane;
     int32_t run;             // bytes of a plane's copy
     int32_t ndep;            // tiles whose previous step it waits for
-    int32_t dep[20];         // their indices; more than 20: dep[0] is their place in dep_idx
+    int32_t dep[19];         // their indices; more than 19: dep[0] is their place in dep_idx
 };
 static_assert(sizeof(TileRec) == 256, "one load of 8 bytes per lane");
 

@@ -129,9 +129,14 @@ __global__ void k_init(const ChareDev *ch, int nch, int64_t nx, int64_t ny, int6
             const int ghosts_yz = (jp == 0 || jp == C.by + 1) + (kp == 0 || kp == C.bz + 1);
             const int64_t gy = C.y0 + jp + oy, gz = C.z0 + kp + oz;
             double *a0 = C.A[0] + (int64_t)rr * C.pitch, *a1 = C.A[1] + (int64_t)rr * C.pitch;
-            for (int cp = lane; cp < C.pitch; cp += 32) {
+            // padded x index cp of column col; the x+ ghost may lie one past the
+            // row, in column 0 of the next, which that row then leaves alone
+            const bool apart = C.col0 == 4;
+            for (int col = lane; col < C.pitch + (apart ? 1 : 0); col += 32) {
+                const int cp = col - C.col0 + 1;
+                if (col == 0 && apart && rr > 0) continue;
                 double v = 0.0;
-                if (cp <= C.bx + 1 && ghosts_yz + (cp == 0 || cp == C.bx + 1) <= 1) {
+                if (cp >= 0 && cp <= C.bx + 1 && ghosts_yz + (cp == 0 || cp == C.bx + 1) <= 1) {
                     const int64_t gx = C.x0 + cp + ox;
                     if (stencil == OD_STENCIL_2D5) {
                         const bool shell = gx == 0 || gz == 0 || gx == nx + 1 || gz == nz + 1;
@@ -141,8 +146,8 @@ __global__ void k_init(const ChareDev *ch, int nch, int64_t nx, int64_t ny, int6
                     }
                 }
                 v = f64_from(fx_encode(v, base));
-                a0[cp] = v;
-                a1[cp] = v;
+                a0[col] = v;
+                a1[col] = v;
             }
         }
     }
@@ -165,9 +170,10 @@ __global__ void k_tile_recs(const ChareDev *ch, const TileDev *tiles, int64_t nt
         R.k0 = T.k0;
         R.nk = T.nk;
         R.bz = C.bz;
-        R.run = d3 ? (T.nj + 2) * C.pitch * 8 : ((T.ni + 3) & ~1) * 8;
+        R.cell0 = d3 ? C.col0 : C.col0 == 4 ? 2 : 1;
+        R.run = d3 ? (T.nj + 2) * C.pitch * 8 : ((T.ni + R.cell0 + 2) & ~1) * 8;
         const bool low = T.k0 == 0, high = T.k0 + T.nk >= C.bz;  // touches the chare's z faces
-        const int64_t org = d3 ? (int64_t)T.j0 * C.pitch : T.i0;
+        const int64_t org = d3 ? (int64_t)T.j0 * C.pitch : T.i0 + C.col0 - R.cell0;
         const ChareDev *N[6];
         for (int f = 0; f < 6; ++f) N[f] = C.nbr[f] >= 0 ? &ch[C.nbr[f]] : nullptr;
         const ChareDev *X0 = N[OD_FACE_XLO], *X1 = N[OD_FACE_XHI], *Y0 = N[OD_FACE_YLO], *Y1 = N[OD_FACE_YHI],
@@ -182,8 +188,8 @@ __global__ void k_tile_recs(const ChareDev *ch, const TileDev *tiles, int64_t nt
             R.own[p] = C.A[p] + org;
             // y- and z-neighbours share the chare's x extent, so its pitch;
             // z-neighbours its y extent too, so its plane
-            R.xlo[p] = X0 ? X0->A[p] + X0->bx + (d3 ? (int64_t)(T.j0 + 1) * X0->pitch : 0) : nullptr;
-            R.xhi[p] = X1 ? X1->A[p] + 1 + (d3 ? (int64_t)(T.j0 + 1) * X1->pitch : 0) : nullptr;
+            R.xlo[p] = X0 ? X0->A[p] + X0->col0 + X0->bx - 1 + (d3 ? (int64_t)(T.j0 + 1) * X0->pitch : 0) : nullptr;
+            R.xhi[p] = X1 ? X1->A[p] + X1->col0 + (d3 ? (int64_t)(T.j0 + 1) * X1->pitch : 0) : nullptr;
             R.ylo[p] = Y0 ? Y0->A[p] + (int64_t)Y0->by * C.pitch : nullptr;
             R.yhi[p] = Y1 ? Y1->A[p] + C.pitch : nullptr;
             R.zlo[p] = Z0 ? Z0->A[p] + (int64_t)Z0->bz * R.plane + org : nullptr;
@@ -197,7 +203,7 @@ __global__ void k_tile_recs(const ChareDev *ch, const TileDev *tiles, int64_t nt
         R.yhi_plane = Y1 ? Y1->rows * C.pitch : 0;
         const int32_t q0 = dep_ptr[t];
         R.ndep = dep_ptr[t + 1] - q0;
-        for (int d = 0; d < 20; ++d) R.dep[d] = R.ndep > 20 ? q0 : d < R.ndep ? dep_idx[q0 + d] : 0;
+        for (int d = 0; d < 19; ++d) R.dep[d] = R.ndep > 19 ? q0 : d < R.ndep ? dep_idx[q0 + d] : 0;
         rec[t] = R;
     }
 }
@@ -209,17 +215,17 @@ __device__ __forceinline__ int64_t face_offset(const ChareDev &C, int f, int q, 
     const int64_t plane = (int64_t)C.rows * pitch;
     if (f < 2) {
         const int k = q / by, j = q - k * by;
-        const int col = f == OD_FACE_XLO ? (ghost ? 0 : 1) : (ghost ? bx + 1 : bx);
+        const int col = C.col0 + (f == OD_FACE_XLO ? (ghost ? -1 : 0) : (ghost ? bx : bx - 1));
         return (k + 1) * plane + (int64_t)(j + r0) * pitch + col;
     }
     if (f < 4) {  // (3D only: a 2D chare has no y faces)
         const int k = q / bx, i = q - k * bx;
         const int row = f == OD_FACE_YLO ? (ghost ? 0 : 1) : (ghost ? by + 1 : by);
-        return (k + 1) * plane + (int64_t)row * pitch + i + 1;
+        return (k + 1) * plane + (int64_t)row * pitch + C.col0 + i;
     }
     const int j = q / bx, i = q - j * bx;
     const int pl = f == OD_FACE_ZLO ? (ghost ? 0 : 1) : (ghost ? bz + 1 : bz);
-    return (int64_t)pl * plane + (int64_t)(j + r0) * pitch + i + 1;
+    return (int64_t)pl * plane + (int64_t)(j + r0) * pitch + C.col0 + i;
 }
 
 // Per-chare path, A4: new boundary planes of parity p -> contiguous send
@@ -327,7 +333,7 @@ __global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t
             for (int u = 0; u < kIoRows; ++u) {
                 const int rr = r0 + u < nrow ? r0 + u : r0;  // past the end: repeat the first row
                 const int k = rr / C.by, j = rr - k * C.by;
-                src[u] = C.A[p] + (k + 1) * plane + (int64_t)(j + C.row0) * C.pitch + 1;
+                src[u] = C.A[p] + (k + 1) * plane + (int64_t)(j + C.row0) * C.pitch + C.col0;
                 dst[u] = g + ((C.z0 + k) * ny + C.y0 + j) * nx + C.x0;
             }
             for (int i = lane; i < bx; i += 32) {
@@ -368,7 +374,7 @@ __global__ void k_scatter(const ChareDev *ch, int nch, int p, int64_t nx, int64_
             for (int u = 0; u < kIoRows; ++u) {
                 const int rr = r0 + u < nrow ? r0 + u : r0;  // past the end: repeat the first row
                 const int k = rr / C.by, j = rr - k * C.by;
-                dst[u] = C.A[p] + (k + 1) * plane + (int64_t)(j + C.row0) * C.pitch + 1;
+                dst[u] = C.A[p] + (k + 1) * plane + (int64_t)(j + C.row0) * C.pitch + C.col0;
                 src[u] = g + ((C.z0 + k) * ny + C.y0 + j) * nx + C.x0;
             }
             for (int i = lane; i < bx; i += 32) {
@@ -420,8 +426,8 @@ __global__ void k_refit(const ChareDev *ch, int nch, int p, int64_t nx, int64_t 
             const bool inside = j >= 0 && j < C.by && k >= 0 && k < C.bz;
             double *a = C.A[p] + (int64_t)rr * C.pitch, *b = C.A[p ^ 1] + (int64_t)rr * C.pitch;
             for (int cp = lane; cp < C.pitch; cp += 32) {
-                if (inside && cp >= 1 && cp <= C.bx) {
-                    a[cp] = f64_from(fx_encode(g[((C.z0 + k) * ny + C.y0 + j) * nx + C.x0 + cp - 1], to));
+                if (inside && cp >= C.col0 && cp < C.col0 + C.bx) {
+                    a[cp] = f64_from(fx_encode(g[((C.z0 + k) * ny + C.y0 + j) * nx + C.x0 + cp - C.col0], to));
                 } else {
                     a[cp] = f64_from(fx_encode(fx_decode(f64_bits(a[cp]), from), to));
                     b[cp] = f64_from(fx_encode(fx_decode(f64_bits(b[cp]), from), to));

@@ -354,7 +354,8 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
                 h.x0 = p.ex[cx]; h.bx = (int32_t)(p.ex[cx + 1] - p.ex[cx]);
                 h.y0 = p.ey[cy]; h.by = (int32_t)(p.ey[cy + 1] - p.ey[cy]);
                 h.z0 = p.ez[cz]; h.bz = (int32_t)(p.ez[cz + 1] - p.ez[cz]);
-                h.pitch = round_up(h.bx + 2, 2);
+                h.col0 = h.bx % 4 == 0 ? 4 : 1;
+                h.pitch = h.bx % 4 == 0 ? h.bx + 4 : round_up(h.bx + 2, 2);
                 h.rows = p.stencil == OD_STENCIL_2D5 ? 1 : h.by + 2;
                 h.row0 = p.stencil == OD_STENCIL_2D5 ? 0 : 1;
                 h.nbr[OD_FACE_XLO] = cx > 0 ? (int32_t)(c - 1) : -1;
@@ -576,7 +577,7 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     p.off_order = take(p.order.size() * sizeof(int32_t));
     p.off_rec = take(p.amode == kDefaultArith ? p.tiles.size() * sizeof(TileRec) : 0);
     for (auto &h : p.ch) {
-        size_t a_bytes = (size_t)(h.bz + 2) * (size_t)h.rows * (size_t)h.pitch * 8;
+        size_t a_bytes = (size_t)(h.bz + 2) * (size_t)h.rows * (size_t)h.pitch * 8 + 32;  // the last row's x+ ghost
         size_t f_bytes = (size_t)h.foff[6] * 8;
         for (int s = 0; s < 2; ++s) h.offA[s] = take(a_bytes);
         h.offSend = take(f_bytes);

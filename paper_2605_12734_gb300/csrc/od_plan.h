@@ -29,7 +29,7 @@ inline int32_t kernel_mode(int32_t arith, bool words) { return words && arith ==
 struct HostChare {
     int32_t cx, cy, cz;
     int64_t x0, y0, z0;
-    int32_t bx, by, bz, pitch;
+    int32_t bx, by, bz, pitch, col0;
     int32_t rows, row0;             // plane layout (see ChareDev)
     int32_t nbr[6];
     int32_t foff[7];

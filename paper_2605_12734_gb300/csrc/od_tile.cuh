@@ -188,7 +188,7 @@ __device__ __forceinline__ Arith arith_setup(const KArgs &a, const KArgs &g) {
 // Where a 3D fused tile reads the faces of its neighbours (source parity),
 // prepared once per tile by thread 0 in shared memory:
 //   x-/x+: the neighbour's column next to the face, cell (row, plane) at
-//          x? + (plane+1)*x?_plane + row*x?_pitch (padded coordinates)
+//          x? + (plane+1)*x?_plane + row*x?_pitch (padded rows)
 //   y-/y+: the neighbour's row next to the face in padded plane q at
 //          y? + q*y?_plane (same x extent, so the same pitch)
 //   z-/z+: the neighbour's plane next to the face, the tile's rows (same x
@@ -267,6 +267,8 @@ __device__ __forceinline__ bool run_tile(const KArgs &a, int tile_id, int sp, Ri
     const double *__restrict__ src = C.A[sp] + (size_t)j0 * pitch;
     double *__restrict__ dst = C.A[dp] + (size_t)j0 * pitch;
     const uint32_t row_bytes = (uint32_t)pitch * 8u;
+    const int col0 = C.col0;
+    const uint32_t lead = col0 == 4 ? 2u : 0u;
     const uint32_t run_bytes = (uint32_t)(nj + 2) * row_bytes;  // one plane's rows
     const int S = g.stages, SD = g.stage_doubles;
     const int kb = T.k0 - 1, ke = T.k0 + T.nk;  // planes kb..ke are loaded
@@ -297,12 +299,14 @@ __device__ __forceinline__ bool run_tile(const KArgs &a, int tile_id, int sp, Ri
                 first = 1;
             }
             if (FUSED && computed && pi->yhi) {
-                bulk_g2s(slot_p + (size_t)(nj + 1) * pitch, pi->yhi + (size_t)(p + 1) * pi->yhi_plane, row_bytes,
-                         bar);
+                // (with the ghosts apart, its first two words hold row nj's x+
+                // ghost, this chare's)
+                bulk_g2s(slot_p + (size_t)(nj + 1) * pitch + lead, pi->yhi + (size_t)(p + 1) * pi->yhi_plane + lead,
+                         row_bytes - 8u * lead, bar);
                 last = nj;
             }
             bulk_g2s(slot_p + (size_t)first * pitch, row0 + (size_t)first * pitch,
-                     (uint32_t)(last - first + 1) * row_bytes, bar);
+                     (uint32_t)(last - first + 1) * row_bytes + (last == nj ? 8u * lead : 0u), bar);
         }
     };
     int issued_hi = kb - 1;  // highest plane issued so far (same value in every thread)
@@ -324,12 +328,12 @@ __device__ __forceinline__ bool run_tile(const KArgs &a, int tile_id, int sp, Ri
             for (int f = 0; f < 6; ++f) {
                 const int n = C.nbr[f];
                 const ChareDev *N = n >= 0 ? &a.ch[n] : nullptr;
-                if (f == OD_FACE_XLO) {  // its column bx_n
-                    pi->xlo = N ? N->A[sp] + N->bx : nullptr;
+                if (f == OD_FACE_XLO) {  // its last column
+                    pi->xlo = N ? N->A[sp] + N->col0 + N->bx - 1 : nullptr;
                     pi->xlo_pitch = N ? N->pitch : 0;
                     pi->xlo_plane = N ? (N->by + 2) * N->pitch : 0;
-                } else if (f == OD_FACE_XHI) {  // its column 1
-                    pi->xhi = N ? N->A[sp] + 1 : nullptr;
+                } else if (f == OD_FACE_XHI) {  // its first column
+                    pi->xhi = N ? N->A[sp] + N->col0 : nullptr;
                     pi->xhi_pitch = N ? N->pitch : 0;
                     pi->xhi_plane = N ? (N->by + 2) * N->pitch : 0;
                 } else if (f == OD_FACE_YLO) {  // its row by_n, when the tile's first halo row is the ghost row
@@ -364,7 +368,7 @@ __device__ __forceinline__ bool run_tile(const KArgs &a, int tile_id, int sp, Ri
         const int q0 = tid + m * NT;
         const int q = q0 < ncell ? q0 : 0;
         const int j = q / bx, i = q - j * bx;
-        rf[m] = (j + 1) * pitch + i + 1;
+        rf[m] = (j + 1) * pitch + col0 + i;
     }
 
     // x-halo patches of a plane (fused only): item t < 2*nj is row t % nj of
@@ -385,7 +389,7 @@ __device__ __forceinline__ bool run_tile(const KArgs &a, int tile_id, int sp, Ri
     };
     auto patch_dst = [&](int t) -> int {
         const bool hi = t >= nj;
-        return ((hi ? t - nj : t) + 1) * pitch + (hi ? bx + 1 : 0);
+        return ((hi ? t - nj : t) + 1) * pitch + col0 + (hi ? bx : -1);
     };
 
     // Planes k-1, k and k+1 must be resident while plane k is computed, so a
@@ -500,10 +504,10 @@ static __device__ __noinline__ double update2d_slow_fx(const double *sd, const d
 // (nx, 1, ny): a chare's 2D rows are its planes, one row each, so A is the
 // padded 2D block and plane k (interior row k) starts at (k+1)*pitch.  A tile
 // is one row segment, columns [i0, i0+ni), over planes [k0, k0+nk).  Per
-// plane one bulk copy brings columns i0 .. i0+ni+1 (the segment plus its
-// x-halo, rounded up to an even count; i0 and pitch are even, so the copy
-// starts 16-byte aligned) into a ring slot; slot offset r = i+1 holds column
-// i0+i+1, i.e. the tile's cell i.
+// plane one bulk copy brings the segment plus its x-halo, an even count from one
+// or two words before its first cell (column 1 or 4: the copy starts 16-byte
+// aligned, as i0 and pitch are even) into a ring slot, whose offset cell0 + i
+// then holds the tile's cell i.
 // The update reads W = slot[r-1], E = slot[r+1] of plane k, S = plane k-1,
 // N = plane k+1 at r, summed in that order and divided by 4.
 // The 2D update of one cell in arithmetic mode AM (m as in update_cell).
@@ -546,9 +550,10 @@ __device__ __forceinline__ bool run_tile_2d(const KArgs &a, int tile_id, int sp,
     const int plane = pitch;
     const int dp = sp ^ 1;
     const int i0 = T.i0, ni = T.ni;
-    const double *__restrict__ src = C.A[sp] + i0;  // column i0 of the lower ghost row
-    double *__restrict__ dst = C.A[dp] + i0;
-    const uint32_t run_bytes = (uint32_t)((ni + 3) & ~1) * 8u;
+    const int cell0 = C.col0 == 4 ? 2 : 1, org = i0 + C.col0 - cell0;
+    const double *__restrict__ src = C.A[sp] + org;  // the copy's first word in the lower ghost row
+    double *__restrict__ dst = C.A[dp] + org;
+    const uint32_t run_bytes = (uint32_t)((ni + cell0 + 2) & ~1) * 8u;
     const int S = g.stages, SD = g.stage_doubles;
     const int kb = T.k0 - 1, ke = T.k0 + T.nk;
     const int tid = threadIdx.x;
@@ -575,15 +580,15 @@ __device__ __forceinline__ bool run_tile_2d(const KArgs &a, int tile_id, int sp,
         const int f = tid < 2 ? tid : tid + 2, n = C.nbr[f];
         const ChareDev *N = n >= 0 ? &a.ch[n] : nullptr;
         if (f == OD_FACE_XLO) {  // its column bx_n, when the segment starts at the chare's edge
-            pi->xlo = N && i0 == 0 ? N->A[sp] + N->bx : nullptr;
+            pi->xlo = N && i0 == 0 ? N->A[sp] + N->col0 + N->bx - 1 : nullptr;
             pi->xlo_plane = N ? N->pitch : 0;
         } else if (f == OD_FACE_XHI) {  // its column 1
-            pi->xhi = N && i0 + ni == bx ? N->A[sp] + 1 : nullptr;
+            pi->xhi = N && i0 + ni == bx ? N->A[sp] + N->col0 : nullptr;
             pi->xhi_plane = N ? N->pitch : 0;
         } else if (f == OD_FACE_ZLO) {  // its row bz_n (same x extent, same pitch)
-            pi->zlo = N && kb < 0 ? N->A[sp] + (size_t)N->bz * plane + i0 : nullptr;
+            pi->zlo = N && kb < 0 ? N->A[sp] + (size_t)N->bz * plane + org : nullptr;
         } else {  // its row 1
-            pi->zhi = N && ke >= bz ? N->A[sp] + plane + i0 : nullptr;
+            pi->zhi = N && ke >= bz ? N->A[sp] + plane + org : nullptr;
         }
     }
     if (FUSED) __syncthreads();  // the pull info
@@ -599,16 +604,16 @@ __device__ __forceinline__ bool run_tile_2d(const KArgs &a, int tile_id, int sp,
 #pragma unroll
     for (int m = 0; m < CPT; ++m) {
         const int q0 = tid + m * NT;
-        rf[m] = (q0 < ni ? q0 : 0) + 1;
+        rf[m] = (q0 < ni ? q0 : 0) + cell0;
     }
-    // x-halo patches (fused only): thread 0 the x- ghost (slot offset 0),
-    // thread 1 the x+ ghost (offset ni + 1) of a computed row
+    // x-halo patches (fused only): thread 0 the x- ghost (before the
+    // first cell), thread 1 the x+ ghost (after the last) of a computed row
     auto patch_src = [&](int p) -> const double * {
         if (!FUSED || tid > 1) return nullptr;
         const double *base = tid ? pi->xhi : pi->xlo;
         return base ? base + (size_t)(p + 1) * (tid ? pi->xhi_plane : pi->xlo_plane) : nullptr;
     };
-    const int patch_dst = tid ? ni + 1 : 0;
+    const int patch_dst = tid ? cell0 + ni : cell0 - 1;
 
     bool fail = !mbar_wait_bounded(ring.bars + slot(kb), phase(kb), g.spin_ns);
     if (!fail) fail = !mbar_wait_bounded(ring.bars + slot(kb + 1), phase(kb + 1), g.spin_ns);

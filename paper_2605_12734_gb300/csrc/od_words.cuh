@@ -81,6 +81,7 @@ struct WordsShared {
         int32_t plane;   // doubles from one destination plane to the next
         int32_t pitch;   // doubles from one row to the next
         int32_t bx, n;   // cells of a row, cells of a plane of the tile
+        int32_t cell0;   // slot offset of a row's first cell
         int32_t nk;      // planes to compute
         int32_t tile;    // -1: no more tiles
         int32_t done;    // what its step counter says when it is done (persistent)
@@ -141,15 +142,16 @@ __device__ __forceinline__ uint32_t count_acq_rel(uint32_t *p) {
 // share packed binary32 operations.  The window is checked once for all of
 // them; the rare plane that fails it has the failing cells redone with IEEE
 // operations, out of line.
-template <int CPT, int ST>
+// N: how many of the CPT cells to do, the first ones.
+template <int CPT, int ST, int N = CPT>
 __device__ __forceinline__ void words_plane(const double *sd, const double *sc, const double *su, double *dpl,
                                             const int (&rf)[CPT], int pitch, uint32_t e0) {
     constexpr bool k3D = ST == OD_STENCIL_3D7;
-    constexpr int W = CPT == 1 ? 1 : 2;
+    constexpr int W = N == 1 ? 1 : 2;
     // bits of every operand's high word, and the lowest top bit of a quotient
     uint32_t any = e0 == 0u ? kFxEnd : 0u, low = 0xFFFFFFFFu;
 #pragma unroll
-    for (int m = 0; m < CPT; m += W) {
+    for (int m = 0; m < N; m += W) {
         uint64_t F[2], b[2][4];
         uint32_t z[2];
 #pragma unroll
@@ -196,7 +198,7 @@ __device__ __forceinline__ void words_plane(const double *sd, const double *sc, 
     }
     if (any >= kFxEnd || low < 20u) {
 #pragma unroll
-        for (int m = 0; m < CPT; ++m) {
+        for (int m = 0; m < N; ++m) {
             const int r = rf[m];
             uint64_t x = f64_bits(sc[r - 1]) | f64_bits(sc[r + 1]) | f64_bits(sd[r]) | f64_bits(su[r]);
             if (k3D) x |= f64_bits(sc[r - pitch]) | f64_bits(sc[r + pitch]);
@@ -228,19 +230,21 @@ __device__ __forceinline__ void words_compute(const KArgs &a, WordsShared &sh, c
         if (tile < 0) break;
         const int pitch = sh.t[i].pitch, plane = sh.t[i].plane;
         int rf[CPT];
+        int busy = 2;  // two cells a thread: how many cells a lane has that are not past the tile's end in the whole warp
         {
-            const int bx = sh.t[i].bx, nc = sh.t[i].n;
+            const int bx = sh.t[i].bx, nc = sh.t[i].n, cell0 = sh.t[i].cell0;
 #pragma unroll
             for (int m = 0; m < CPT; ++m) {
                 const int q0 = tid + m * NT;
                 const int q = q0 < nc ? q0 : 0;
                 if (ST == OD_STENCIL_3D7) {
                     const int j = q / bx;
-                    rf[m] = (j + 1) * pitch + (q - j * bx) + 1;
+                    rf[m] = (j + 1) * pitch + cell0 + (q - j * bx);
                 } else {
-                    rf[m] = q + 1;
+                    rf[m] = cell0 + q;
                 }
             }
+            if (CPT == 2) busy = (nc - (tid & ~31) + NT - 1) / NT;
         }
         // the planes below the first computed one and that one
         uint64_t *held_d = &sh.empty[sl];  // the slots of planes k-1 and k
@@ -255,7 +259,13 @@ __device__ __forceinline__ void words_compute(const KArgs &a, WordsShared &sh, c
             advance();
             const double *su = ring + (size_t)sl * SD;
             if (!(ok = wait_phase(&sh.ready[sl], ph, &sh.stop, limit))) break;
-            words_plane<CPT, ST>(sd, sc, su, dpl, rf, pitch, e0);
+            // In the shapes of two cells a thread, which narrow planes get, a
+            // warp past the plane's end has nothing to do and one in its last
+            // part one cell (5195 x 7129 in 83-cell rows: 0.392 / 0.318 ms a
+            // step).  With four cells the second form spills: 32^3 chares ran
+            // 0.60 instead of 0.48 ms.
+            if (CPT != 2 || busy > 1) words_plane<CPT, ST>(sd, sc, su, dpl, rf, pitch, e0);
+            else if (busy > 0) words_plane<CPT, ST, CPT == 2 ? 1 : CPT>(sd, sc, su, dpl, rf, pitch, e0);
             __syncwarp();
             if (lane == 0) mbar_arrive(held_d);
             held_d = held_c;
@@ -302,7 +312,7 @@ __device__ __forceinline__ HaloItem halo_item(const TileRec &R, int sp, int t) {
     const double *base = hi ? R.xhi[sp] : R.xlo[sp];
     h.plane = hi ? R.xhi_plane : R.xlo_plane;
     if (base) h.src = base + (int64_t)j * (hi ? R.xhi_pitch : R.xlo_pitch);
-    h.off = ST == OD_STENCIL_3D7 ? (j + 1) * R.pitch + (hi ? R.bx + 1 : 0) : (hi ? R.cells + 1 : 0);
+    h.off = ST == OD_STENCIL_3D7 ? (j + 1) * R.pitch + R.cell0 + (hi ? R.bx : -1) : R.cell0 + (hi ? R.cells : -1);
     return h;
 }
 
@@ -351,13 +361,13 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
             const TileRec &N = sh.rec[n & 1u];
             stage = 4;
             if (PERSIST) {
-                if (N.ndep <= 20) seen = lane < N.ndep ? ld_acquire(a.epoch + N.dep[lane]) : INT32_MAX;
+                if (N.ndep <= 19) seen = lane < N.ndep ? ld_acquire(a.epoch + N.dep[lane]) : INT32_MAX;
                 stage = 3;
             }
         } else if (stage == 3) {
             // once only: further looks wait until the tile's turn, so that
             // they do not hold up the planes of the current one
-            stage = sh.rec[n & 1u].ndep <= 20 && __all_sync(0xFFFFFFFFu, seen >= nr) ? 4 : 5;
+            stage = sh.rec[n & 1u].ndep <= 19 && __all_sync(0xFFFFFFFFu, seen >= nr) ? 4 : 5;
         }
     };
     for (uint32_t n = 0;; ++n) {
@@ -374,7 +384,7 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
             // published by its compute warps).
             if (stage != 4) {
                 const int nd = R.ndep;
-                const int32_t *more = nd > 20 ? a.dep_idx + R.dep[0] : nullptr;
+                const int32_t *more = nd > 19 ? a.dep_idx + R.dep[0] : nullptr;
                 int q = lane;
                 uint64_t t0 = 0;
                 for (uint32_t k = 1;; ++k) {
@@ -423,6 +433,7 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
             t.plane = plane;
             t.pitch = R.pitch;
             t.bx = R.bx;
+            t.cell0 = R.cell0;
             t.n = R.cells;
             t.nk = R.nk;
             t.tile = tile;
@@ -457,8 +468,12 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
                     bytes -= row_bytes;
                 }
                 if (FUSED && computed && yhi) {
-                    bulk_g2s(to + (size_t)(R.rows + 1) * R.pitch, yhi + (int64_t)(p + 1) * R.yhi_plane, row_bytes, bar);
-                    bytes -= row_bytes;
+                    // (with the ghosts apart, its first two words hold the
+                    // last row's x+ ghost, this chare's)
+                    const uint32_t lead = R.cell0 == 4 ? 2u : 0u;
+                    bulk_g2s(to + (size_t)(R.rows + 1) * R.pitch + lead, yhi + (int64_t)(p + 1) * R.yhi_plane + lead,
+                             row_bytes - 8u * lead, bar);
+                    bytes -= row_bytes - 8u * lead;
                 }
                 bulk_g2s(at, row0, bytes, bar);
             } else {

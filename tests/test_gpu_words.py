@@ -109,7 +109,7 @@ def test_faces_fed_from_outside(od, path):
 
 
 @pytest.mark.parametrize("kw", [
-    dict(cuts=([0, 4, 260], [0, 128], [0, 3])),                       # a tile that reads more than 20 others
+    dict(cuts=([0, 4, 260], [0, 128], [0, 3])),                       # a tile that reads more than 19 others
     dict(cuts=([0, 1, 2, 260], [0, 1, 128], [0, 1, 3]), tile_z=1),     # single cells, rows and planes
     dict(split=(2, 2, 1), stages=3, tile_z=2), dict(split=(2, 2, 1), stages=8, tile_z=1),
     dict(split=(3, 2, 3), threads=512, cells_per_thread=1), dict(split=(1, 4, 1), threads=256, cells_per_thread=8),
