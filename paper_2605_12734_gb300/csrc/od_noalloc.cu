@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kBlock, 4)
     const uint32_t k0 = blockIdx.y * chunk, k1 = min(k0 + chunk, nz);
     for (uint32_t k = k0; k < k1; ++k) {
         const double *p = src + (size_t)k * sxy;
-        od::tile::words_plane<kCells, OD_STENCIL_3D7>(p, p + sxy, p + 2u * sxy, dst + (size_t)(k + 1u) * sxy, rf,
+        od::tile::words_plane<kCells, OD_STENCIL_3D7, false>(p, p + sxy, p + 2u * sxy, dst + (size_t)(k + 1u) * sxy, rf,
                                                       (int)sx, base);
     }
 }

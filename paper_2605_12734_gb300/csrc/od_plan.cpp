@@ -79,11 +79,11 @@ int32_t stage_doubles_for(int32_t nj, int32_t pitch) {
     return round_up((nj + 2) * pitch, 16);     // keep slots 128-byte aligned
 }
 
-// Tiles and dependency-list entries of the grid with tz planes per tile (the
-// shape, the tile rows and the cuts of p), as build_plan lays them out.
-static void count_tiles(const Plan &p, int32_t tz, int64_t *ntiles, int64_t *ndeps) {
+// Tiles and dependency-list entries of the grid with cap cells per tile plane
+// and tz planes per tile (the tile rows and the cuts of p), as build_plan lays
+// them out.
+static void count_tiles(const Plan &p, int64_t cap, int32_t tz, int64_t *ntiles, int64_t *ndeps) {
     const bool d3 = p.stencil == OD_STENCIL_3D7;
-    int64_t cap = (int64_t)p.threads * p.cpt;
     if (!d3 && p.tile_y > 0) cap = std::min<int64_t>(cap, p.tile_y);
     auto parts = [](int64_t n, int64_t most) { return (n + std::min(n, most) - 1) / std::min(n, most); };
     const size_t nx = p.ex.size() - 1, ny = p.ey.size() - 1, nz = p.ez.size() - 1;
@@ -139,26 +139,47 @@ static size_t table_bytes(int64_t nt, int64_t nd) {
            a((size_t)std::max<int64_t>(1, nd) * 4) + a((size_t)nt * 4) + a((size_t)nt * sizeof(TileRec));
 }
 
+// Whether a context's sweep over words runs 256 x 4 where the plan, not told a
+// shape, reports 128 x 4: both use every lane and 128 x 4 holds eight rows or
+// fewer, so 256 x 4 copies half the halo rows and has half the producers (512^3
+// in 64^3 / 128^3 chares 0.444 / 0.465 ms a step with 128 x 4, 0.427 / 0.425
+// with 256 x 4; 32-cell rows 0.460 / 0.50).  Large grids only, whose tiles are
+// still many.
+static bool words_wide(const Plan &p) {
+    if (p.stencil != OD_STENCIL_3D7 || p.threads != 128 || p.cpt != 4 || p.tile_y > 0 ||
+        p.nx * p.ny * p.nz < (1 << 24))
+        return false;
+    for (size_t e = 1; e < p.ex.size(); ++e) {
+        const int64_t w = p.ex[e] - p.ex[e - 1];
+        if (w < 64 || 512 % w != 0) return false;
+        for (size_t b = 1; b < p.ey.size(); ++b)
+            if ((p.ey[b] - p.ey[b - 1]) % (1024 / w) != 0) return false;
+    }
+    return true;
+}
+
 // Planes (2D: rows) per tile that a context's sweep over words runs with when
 // none is asked for.  Tall tiles copy fewer halo planes, but a grid of few
 // tiles leaves CTAs idle and makes every step wait for its slowest tile; about
 // two tiles per resident CTA keep the CTAs busy across steps.  So: the tallest
-// that gives 1800 tiles, 4 where none does, 2 where that leaves fewer than
-// 800.  Measured, us a step with 32 planes and with the rule's: 64^3 in 8
+// that gives 1800 tiles (900 of 256 threads), 4 where none does, 2 where that
+// leaves fewer than 800.  Measured, us a step with 32 planes and with the rule's: 64^3 in 8
 // chares 24.6 / 8.0, 100^3 in 8 21.0 / 11.4, 128^3 in 64 26.5 / 13.6, 203^3 in
 // 27 45.6 / 35.4, 256^3 in 64 72.4 / 60.8; 300^3 in 216 98.2 with 32 (2160
 // tiles), 101.6 with 16.  2D: 96 x 64 in 4 20.0 / 4.9, 1000 x 777 in 16 18.1 /
 // 8.4, 2048^2 in 16 26.0 / 13.4, 5000 x 3000 in 16 49.7 / 44.0, 8192^2 in 256
 // 169 / 165 (64 rows), 16384^2 in 1024 678 / 662.
-static int32_t words_tile_z(const Plan &p) {
+static int32_t words_tile_z(const Plan &p, int32_t threads, int32_t cpt) {
     const bool d3 = p.stencil == OD_STENCIL_3D7;
     auto tiles_with = [&](int32_t tz) {
         int64_t nt = 0, nd = 0;
-        count_tiles(p, tz, &nt, &nd);
+        count_tiles(p, (int64_t)threads * cpt, tz, &nt, &nd);
         return nt;
     };
     int32_t tz = d3 ? 32 : 64;
-    while (tz > 4 && tiles_with(tz) < 1800) tz /= 2;
+    // (256 threads and more: half as many CTAs are resident)
+    const int64_t enough = threads >= 256 ? 900 : 1800;
+    while (tz > 4 && tiles_with(tz) < enough) tz /= 2;
     return tz == 4 && tiles_with(4) < 800 ? 2 : tz;
 }
 
@@ -382,9 +403,14 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     p.bytes_per_step = 16.0 * (double)p.cells + 16.0 * (double)p.face_internal +
                        8.0 * (double)p.face_dirichlet;
 
-    // a context runs the default arithmetic with its own planes per tile
-    const int32_t run_z = cfg->tile_z == 0 && p.amode == kDefaultArith ? words_tile_z(p) : 0;
-    const int32_t tile_z = cfg->tile_z > 0 ? cfg->tile_z : running && run_z ? run_z : 32;
+    // a context runs the default arithmetic with its own shape and planes per
+    // tile where none are asked for
+    const bool words = p.amode == kDefaultArith;
+    const bool wide = words && auto_shape && fill_gpu && words_wide(p);
+    const int32_t run_threads = wide ? 256 : p.threads;
+    const int32_t run_z = cfg->tile_z > 0 ? cfg->tile_z : words ? words_tile_z(p, run_threads, p.cpt) : 32;
+    const int32_t tile_z = cfg->tile_z > 0 ? cfg->tile_z : running ? run_z : 32;
+    if (running) p.threads = run_threads;
 
     // tiles: full rows, balanced row slabs and plane chunks
     std::vector<int32_t> js, jl, ks, kl;
@@ -585,10 +611,10 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
         h.offRecv[1] = take(f_bytes);
     }
     p.arena_bytes = at;
-    if (!running && run_z && run_z != tile_z) {
+    if (!running && (run_z != tile_z || run_threads != p.threads)) {
         // the arena also holds the tables of the tiles a context will run with
         int64_t nt = 0, nd = 0;
-        count_tiles(p, run_z, &nt, &nd);
+        count_tiles(p, (int64_t)run_threads * p.cpt, run_z, &nt, &nd);
         const size_t mine = table_bytes((int64_t)p.tiles.size(), (int64_t)p.dep_idx.size()), run = table_bytes(nt, nd);
         if (run > mine) p.arena_bytes += run - mine;
     }

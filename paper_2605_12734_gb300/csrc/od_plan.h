@@ -72,8 +72,8 @@ od_status build_plan(const od_config *cfg, Plan *plan, std::string *err);
 // when fill_gpu is false (a batch of many jobs fills the GPU, so a job's own
 // tile count does not count against a shape), as the serving loop does.
 // running: the plan that a context runs, whose planes per tile follow its size
-// when none are asked for; otherwise the plan as it is reported, with 32, in
-// an arena that holds either.
+// when none are asked for (and whose CTA shape may be a larger one); otherwise
+// the plan as it is reported, with 32, in an arena that holds either.
 od_status build_plan(const od_config *cfg, Plan *plan, std::string *err, bool fill_gpu, bool running = false);
 
 // Ring-slot size for a tile of `nj` rows in a chare of row pitch `pitch`

@@ -135,15 +135,71 @@ __device__ __forceinline__ uint32_t count_acq_rel(uint32_t *p) {
 
 // ---------------------------------------------------------------- compute warps
 
+// The cells of a warp's plane that have an operand or a quotient outside the
+// window (`rare`: this lane may have some), with IEEE operations: they are
+// numbered over the warp and dealt to its lanes, so that a few scattered ones
+// take one call instead of one for each of a thread's cells (the first step
+// from a uniform random field, 2 % of the cells, 512^3 in 64^3 chares: 1.31 ms
+// without, 1.07 with it; 40 steps from a cold 200^3 field 3.88 and 3.48).
+// Out of line: 64^3 chares in 256 x 4 0.427 ms a step, inlined 0.433.
+template <int N>
+struct Offsets {
+    int r[N];
+};
+
+template <int ST, int N>
+static __device__ __noinline__ void words_redo(const double *sd, const double *sc, const double *su, double *dpl,
+                                               Offsets<N> rf, int pitch, uint32_t e0, bool rare) {
+    constexpr bool k3D = ST == OD_STENCIL_3D7;
+    __shared__ int32_t lists[16][32];  // one per warp of a CTA of up to 512 compute threads
+    int32_t *list = lists[threadIdx.x >> 5];
+    const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+    uint32_t number[N], total = 0;
+#pragma unroll
+    for (int m = 0; m < N; ++m) {
+        const int r = rf.r[m];
+        bool bad = rare;
+        if (bad && e0 != 0u) {
+            const uint64_t w = f64_bits(sc[r - 1]), e = f64_bits(sc[r + 1]), d = f64_bits(sd[r]), u = f64_bits(su[r]);
+            uint64_t x = w | e | d | u, sum = w + e + d + u;
+            if (k3D) {
+                const uint64_t v = f64_bits(sc[r - pitch]), n = f64_bits(sc[r + pitch]);
+                x |= v | n;
+                sum += v + n;
+            }
+            // a quotient below 2^52 needs a sum below that times the divisor;
+            // the margin covers the roundings on the way (a cell redone in
+            // vain gets the same bits)
+            bad = (uint32_t)(x >> 32) >= kFxEnd || (sum != 0u && sum < ((k3D ? 6ull : 4ull) << 52) + 4096u);
+        }
+        const uint32_t mask = __ballot_sync(0xFFFFFFFFu, bad);
+        number[m] = bad ? total + (uint32_t)__popc(mask & below) : 0xFFFFFFFFu;
+        total += (uint32_t)__popc(mask);
+    }
+#pragma unroll 1
+    for (uint32_t base = 0; base < total; base += 32u) {
+#pragma unroll
+        for (int m = 0; m < N; ++m)
+            if (number[m] - base < 32u) list[number[m] - base] = rf.r[m];
+        __syncwarp();
+        if (base + lane < total) {
+            const int r = list[lane];
+            dpl[r] = k3D ? update_slow_fx(sd + r, sc + r, su + r, pitch, e0) : update2d_slow_fx(sd + r, sc + r, su + r, e0);
+        }
+        __syncwarp();
+    }
+}
+
 // One thread's cells of plane k, whose planes below, of and above it lie in the
 // ring slots sd, sc and su: cell m is q = tid + m*NT of the tile's plane,
 // row-major, at slot offset rf[m] (a cell past the end repeats cell 0: the
 // same value to the same place).  Cells are worked on in pairs, whose roundings
 // share packed binary32 operations.  The window is checked once for all of
-// them; the rare plane that fails it has the failing cells redone with IEEE
-// operations, out of line.
-// N: how many of the CPT cells to do, the first ones.
-template <int CPT, int ST, int N = CPT>
+// them; the cells of a plane that fails it are redone with IEEE operations, out
+// of line.  All lanes of a warp call it together.
+// N: how many of the CPT cells to do, the first ones.  DEAL: redo through
+// words_redo (otherwise each lane its own cells).
+template <int CPT, int ST, bool DEAL, int N = CPT>
 __device__ __forceinline__ void words_plane(const double *sd, const double *sc, const double *su, double *dpl,
                                             const int (&rf)[CPT], int pitch, uint32_t e0) {
     constexpr bool k3D = ST == OD_STENCIL_3D7;
@@ -196,7 +252,15 @@ __device__ __forceinline__ void words_plane(const double *sd, const double *sc, 
             low = top < low ? top : low;
         }
     }
-    if (any >= kFxEnd || low < 20u) {
+    const bool rare = any >= kFxEnd || low < 20u;
+    if constexpr (DEAL) {
+        if (__any_sync(0xFFFFFFFFu, rare)) {
+            Offsets<N> o;
+#pragma unroll
+            for (int m = 0; m < N; ++m) o.r[m] = rf[m];
+            words_redo<ST, N>(sd, sc, su, dpl, o, pitch, e0, rare);
+        }
+    } else if (rare) {
 #pragma unroll
         for (int m = 0; m < N; ++m) {
             const int r = rf[m];
@@ -211,6 +275,9 @@ __device__ __forceinline__ void words_plane(const double *sd, const double *sc, 
 
 template <int NT, int CPT, int ST, bool PUBLISH>
 __device__ __forceinline__ void words_compute(const KArgs &a, WordsShared &sh, const double *ring) {
+    // dealing needs a few registers, which only the larger CTAs have to spare
+    // (128 x 4 spills with it: 32^3 chares 0.481 instead of 0.460 ms a step)
+    constexpr bool kDeal = NT >= 256;
     const int tid = threadIdx.x, lane = tid & 31;
     const int S = a.stages, SD = a.stage_doubles;
     const uint32_t e0 = a.fmt->base;
@@ -264,8 +331,8 @@ __device__ __forceinline__ void words_compute(const KArgs &a, WordsShared &sh, c
             // part one cell (5195 x 7129 in 83-cell rows: 0.392 / 0.318 ms a
             // step).  With four cells the second form spills: 32^3 chares ran
             // 0.60 instead of 0.48 ms.
-            if (CPT != 2 || busy > 1) words_plane<CPT, ST>(sd, sc, su, dpl, rf, pitch, e0);
-            else if (busy > 0) words_plane<CPT, ST, CPT == 2 ? 1 : CPT>(sd, sc, su, dpl, rf, pitch, e0);
+            if (CPT != 2 || busy > 1) words_plane<CPT, ST, kDeal>(sd, sc, su, dpl, rf, pitch, e0);
+            else if (busy > 0) words_plane<CPT, ST, kDeal, CPT == 2 ? 1 : CPT>(sd, sc, su, dpl, rf, pitch, e0);
             __syncwarp();
             if (lane == 0) mbar_arrive(held_d);
             held_d = held_c;

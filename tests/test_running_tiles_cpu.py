@@ -36,7 +36,8 @@ def test_arena_holds_the_running_tiles(od, two):
         kw.update(threads=info["threads"], cells_per_thread=info["cells_per_thread"])
         plans = {z: od.plan(*d, tile_z=z, **kw) for z in (2, 4, 8, 16, 32, 64)}
         tz = 64 if two else 32
-        while tz > 4 and plans[tz]["ntiles"] < 1800:
+        enough = 900 if info["threads"] >= 256 else 1800
+        while tz > 4 and plans[tz]["ntiles"] < enough:
             tz //= 2
         if tz == 4 and plans[4]["ntiles"] < 800:
             tz = 2
@@ -44,3 +45,14 @@ def test_arena_holds_the_running_tiles(od, two):
         assert info["ntiles"] == plans[32]["ntiles"]
         assert info["arena_bytes"] == max(plans[32]["arena_bytes"], plans[tz]["arena_bytes"])
     assert finer > 100
+
+
+def test_arena_of_a_wider_running_shape(od):
+    # 64-cell rows: reported 128 x 4, run 256 x 4, whose tables are smaller
+    kw = dict(split=(4, 4, 4))
+    info = od.plan(256, 256, 256, **kw)
+    assert (info["threads"], info["cells_per_thread"]) == (128, 4)
+    wide = od.plan(256, 256, 256, threads=256, cells_per_thread=4, tile_z=16, **kw)
+    assert info["arena_bytes"] >= wide["arena_bytes"]
+    assert info["arena_bytes"] == max(wide["arena_bytes"], od.plan(256, 256, 256, threads=128, cells_per_thread=4,
+                                                                   tile_z=32, **kw)["arena_bytes"])
