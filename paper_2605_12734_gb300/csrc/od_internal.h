@@ -122,7 +122,7 @@ struct KArgs {
     const ChareDev *ch;
     const TileDev *tiles;
     ErrDev *err;
-    int32_t *queue;          // persistent: ticket counter (zeroed per launch)
+    int32_t *queue;          // ticket counter (persistent: zeroed per launch; fused: left at zero)
     int32_t *epoch;          // persistent: steps finished per tile in this launch
     const int32_t *dep_ptr;  // persistent: CSR of the tiles each tile reads
     const int32_t *dep_idx;

@@ -18,7 +18,8 @@ constexpr int32_t kDefaultArith = 12;
 constexpr int32_t kFxMode = 16;  // the tile kernels' mode for mode 12 over such words
 // Resident CTAs per SM of the kernels over words (od_words.cuh): their
 // register budget a thread, for NT compute threads and the producer warp.
-// Measured at 512^3 in 4096 chares (128 x 4): 64 registers 0.489 ms a step,
+// Measured at 512^3 in 4096 chares (128 x 4, rows not yet of whole sectors, which
+// took 64 registers to 0.460): 64 registers 0.489 ms a step,
 // 56 (7 CTAs, a few spills) 0.496, 80 (5 CTAs) 0.60; 32768^2: 56 registers.
 constexpr int words_regs(int cpt, bool d3) { return cpt > 4 ? 112 : d3 ? 64 : 56; }
 constexpr int words_ctas(int nt, int cpt, bool d3) {

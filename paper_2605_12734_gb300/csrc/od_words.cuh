@@ -7,7 +7,7 @@
 // sweep back next -- a CTA barrier on every plane, and one warp delayed each
 // plane by issuing copies and patching the x halo -- would bound this one.
 // Here the CTA is specialised by warp instead: NT compute threads and one
-// producer warp.  The producer takes tiles (tickets on the persistent path),
+// producer warp.  The producer takes tiles (by ticket where its CTA has several),
 // waits for their dependencies, issues the bulk copies of their planes into
 // the ring, patches each landed plane's x halo, and hands the plane over; the
 // compute warps release a slot when they have read it.  No barrier joins the
@@ -27,14 +27,17 @@
 // sweep over doubles, 0.565 that sweep over words, 0.597 this one with a
 // producer that alternates strictly between issuing and finishing planes,
 // 0.541 event-driven, 0.524 with one 256-byte record per tile instead of five
-// dependent table reads, 0.489 with 6 ring slots.  Two-dimensional, 16384^2:
-// 0.76 to 0.67.  What bounds it: at 32^3 chares the traffic (0.456 ms with the
-// roundings left out; 2.58 GB a step, 0.83 of the copy bandwidth) and the ALU
-// pipe (59 % busy) together.  Tried and slower: each thread's own cells of three
-// planes kept in registers (80 registers, five CTAs), publishing a tile from
-// the producer (its fence waits for the whole SM's stores), a full fence after
-// the dependency wait (+6000 cycles a tile), nanosleep in the producer's loop,
-// taking the next ticket earlier than the last plane's issue.
+// dependent table reads, 0.489 with 6 ring slots (0.456 with the roundings left
+// out), 0.460 with rows of whole sectors (od_plan.cpp).  Two-dimensional,
+// 16384^2: 0.76 to 0.65.  What bounds it: at 32^3 chares the traffic (2.50 GB a
+// step, 0.80 of the copy bandwidth) and the ALU pipe (65 % busy, issue 71 %)
+// together; in two dimensions the copy bandwidth (0.99 of it).  A fused step on
+// the same case: 0.553 with a fixed stride of tiles per CTA, 0.480 by ticket.
+// Tried and slower: each thread's own cells of three planes kept in registers
+// (80 registers, five CTAs), publishing a tile from the producer (its fence
+// waits for the whole SM's stores), a full fence after the dependency wait
+// (+6000 cycles a tile), nanosleep in the producer's loop, taking the next
+// ticket earlier than the last plane's issue.
 //
 // Every wait is bounded.  Whoever runs into a limit records the error and
 // raises `stop`, which ends every other wait of the CTA; the producer leaves
@@ -402,8 +405,14 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
     int32_t seen = 0;
     auto look_up = [&](uint32_t n) {  // one stage for tile number n of this CTA
         if (stage == 0) {
-            if (PERSIST) {
-                if (lane == 0) ticket = atomicAdd(a.queue, 1);
+            // Tickets: on the persistent path every tile of every step; in a
+            // fused step those past the grid's, whose CTAs take their own
+            // first (a step of few tiles then waits for no counter).  Each CTA
+            // draws until one is past the end, so the last draw's number is
+            // known, and it leaves the counter at zero for the next launch.
+            if (lane == 0 && (PERSIST || (FUSED && n > 0u && a.tile_count > (int)gridDim.x))) {
+                ticket = atomicAdd(a.queue, 1);
+                if (ticket == (PERSIST ? a.iters * a.ntiles + (int)gridDim.x : a.tile_count) - 1) *a.queue = 0;
             }
             stage = 1;
         } else if (stage == 1) {
@@ -417,7 +426,9 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
                     ntile = a.order ? a.order[pos] : pos;
                 }
             } else {
-                const int64_t tk = (int64_t)blockIdx.x + (int64_t)n * gridDim.x;
+                int64_t tk = (int64_t)blockIdx.x + (int64_t)n * gridDim.x;
+                if (FUSED && n > 0u && a.tile_count > (int)gridDim.x)
+                    tk = (int64_t)gridDim.x + __shfl_sync(0xFFFFFFFFu, ticket, 0);
                 if (tk < a.tile_count) ntile = a.tile_begin + (int)tk;
             }
             if (ntile >= 0) word = reinterpret_cast<const uint64_t *>(a.rec + ntile)[lane];
@@ -645,8 +656,9 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
 
 // NT compute threads and the producer warp (the last one).  FUSED: faces read
 // from the neighbours' arrays; PERSIST: all steps in one launch, tiles by
-// ticket (see k_persistent), otherwise the launch's tiles in turn,
-// gridDim.x apart.  The registers allow words_ctas CTAs per SM (od_plan.h).
+// ticket (see k_persistent).  FUSED alone draws one step's tiles by ticket too;
+// a per-chare launch has its tiles in turn, gridDim.x apart.  The registers
+// allow words_ctas CTAs per SM (od_plan.h).
 template <int NT, int CPT, bool FUSED, bool PERSIST, int ST>
 __global__ void __launch_bounds__(NT + 32, words_ctas(NT, CPT, ST == OD_STENCIL_3D7)) k_words(const KArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];

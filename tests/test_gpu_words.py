@@ -123,6 +123,18 @@ def test_tile_shapes(od, path, kw):
         assert same(s.read(), want)
 
 
+# a fused step draws tickets for the tiles past its resident CTAs (152 SMs x 6 at
+# 128 x 4) and leaves the counter at zero for the next launch of any path
+@pytest.mark.parametrize("tiles", [911, 912, 913, 1823, 1825, 4001])
+def test_fused_tickets(od, tiles):
+    want = oracle.solve(5, 2, tiles, 3, 1, 9)
+    with od.Jacobi3D(5, 2, tiles, split=(1, 1, 1), seed=3, path="fused", tile_z=1, threads=128, cells_per_thread=4) as s:
+        for path, n in (("fused", 3), ("persistent", 2), ("fused_graph", 1), ("fused", 2), ("persistent", 1)):
+            s.set_path(path)
+            s.step(n)
+        assert same(s.read(), want)
+
+
 @pytest.mark.parametrize("kind", ["edges", "tiny", "huge", "infinite"])
 @pytest.mark.parametrize("path", ["persistent", "fused", "per_chare"])
 def test_2d_fields_outside_the_window(od, path, kind):
