@@ -139,23 +139,43 @@ static size_t table_bytes(int64_t nt, int64_t nd) {
            a((size_t)std::max<int64_t>(1, nd) * 4) + a((size_t)nt * 4) + a((size_t)nt * sizeof(TileRec));
 }
 
-// Whether a context's sweep over words runs 256 x 4 where the plan, not told a
-// shape, reports 128 x 4: both use every lane and 128 x 4 holds eight rows or
-// fewer, so 256 x 4 copies half the halo rows and has half the producers (512^3
-// in 64^3 / 128^3 chares 0.444 / 0.465 ms a step with 128 x 4, 0.427 / 0.425
-// with 256 x 4; 32-cell rows 0.460 / 0.50).  Large grids only, whose tiles are
-// still many.
-static bool words_wide(const Plan &p) {
-    if (p.stencil != OD_STENCIL_3D7 || p.threads != 128 || p.cpt != 4 || p.tile_y > 0 ||
-        p.nx * p.ny * p.nz < (1 << 24))
-        return false;
-    for (size_t e = 1; e < p.ex.size(); ++e) {
-        const int64_t w = p.ex[e] - p.ex[e - 1];
-        if (w < 64 || 512 % w != 0) return false;
-        for (size_t b = 1; b < p.ey.size(); ++b)
-            if ((p.ey[b] - p.ey[b - 1]) % (1024 / w) != 0) return false;
-    }
-    return true;
+// Threads and cells a thread with which a context's sweep over words runs where
+// the plan, not told a shape, reports 128 x 2 or 128 x 4 (cells a CTA: 256, 512).
+// A CTA of twice the cells has tiles of twice the rows: half the halo rows
+// copied, half the producers, and from 256 threads on rare cells dealt over the
+// warp; but rows that do not fill its lanes leave more of them idle.  So: twice
+// the cells while that offers no more lanes to the same cells, and 256 x 4 only
+// where 5/8 of its lanes have a cell, and for fused steps, which end in a partial
+// wave, three waves of its tiles.  us a persistent step with
+// 128 x 2 / 128 x 4 / 256 x 4: 100x400x50 in 4 18.3 / 12.5 / 10.9, 128^3 in 64
+// 14.8 / 12.9 / 11.5, 160^3 in 8 24.4 / 18.9 / 17.9, 192^3 in 27 39.8 / 29.7 /
+// 28.4, 400^3 in 1000 341 / 276 / 264; with the last two: 203^3 in 27 34.5 /
+// 33.0, 512^3 in 512 444 / 427, in 4096 460 / 444, 768x512x512 in 300 uneven
+// 767 / 718.  More lanes: 95-cell columns of 100-cell rows (1.05 times) 827 /
+// 826, 72^3 chares (1.09) 690 / 713, 56^3 (1.14) 342 / 369, 36^3 (1.33) 97 / 122.
+// Fused: 512^3 in 4096 480 / 468, 400^3 in 1000 293 / 282; few waves: 128^3 in 8
+// 17.9 / 18.5, 479x128x466 in 15 (1.02 times the lanes) 123 / 132.
+// 24^3 chares fill 9/16: 663 / 634, but a fused step 639 / 658.  Grids under
+// 2^19 cells keep the reported shape (64^3 in 8 chares: 7.6 / 7.8 / 7.4, fused
+// 9.2 / 9.7 / 10.3).
+static void words_shape(const Plan &p, bool fused, int32_t *threads, int32_t *cpt) {
+    if (p.stencil != OD_STENCIL_3D7 || p.threads != 128 || (p.cpt != 2 && p.cpt != 4) || p.tile_y > 0 ||
+        p.nx * p.ny * p.nz < (1 << 19))
+        return;
+    auto lanes = [&](int64_t cap) {  // offered to a plane of the grid's tiles
+        int64_t n = 0;
+        for (size_t a = 1; a < p.ex.size(); ++a)
+            for (size_t b = 1; b < p.ey.size(); ++b) {
+                const int64_t h = p.ey[b] - p.ey[b - 1], rows = std::min(h, cap / (p.ex[a] - p.ex[a - 1]));
+                n += (h + rows - 1) / rows * cap;
+            }
+        return n;
+    };
+    if (*cpt == 2 && lanes(512) <= lanes(256)) *cpt = 4;
+    if (*cpt != 4 || lanes(1024) > lanes(512) || p.nx * p.ny * 8 < lanes(1024) * 5) return;
+    int64_t nt = 0, nd = 0;
+    if (fused) count_tiles(p, 1024, 32, &nt, &nd);
+    if (!fused || nt >= 3 * 3 * 152) *threads = 256;  // three resident CTAs an SM
 }
 
 // Planes (2D: rows) per tile that a context's sweep over words runs with when
@@ -406,11 +426,19 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     // a context runs the default arithmetic with its own shape and planes per
     // tile where none are asked for
     const bool words = p.amode == kDefaultArith;
-    const bool wide = words && auto_shape && fill_gpu && words_wide(p);
-    const int32_t run_threads = wide ? 256 : p.threads;
-    const int32_t run_z = cfg->tile_z > 0 ? cfg->tile_z : words ? words_tile_z(p, run_threads, p.cpt) : 32;
-    const int32_t tile_z = cfg->tile_z > 0 ? cfg->tile_z : running ? run_z : 32;
-    if (running) p.threads = run_threads;
+    auto run_shape = [&](bool fused, int32_t *threads, int32_t *cpt) {  // returns the planes per tile
+        *threads = p.threads;
+        *cpt = p.cpt;
+        if (words && auto_shape && fill_gpu) words_shape(p, fused, threads, cpt);
+        return cfg->tile_z > 0 ? cfg->tile_z : words ? words_tile_z(p, *threads, *cpt) : 32;
+    };
+    int32_t tile_z = cfg->tile_z > 0 ? cfg->tile_z : 32;
+    if (running) {
+        int32_t threads, cpt;
+        tile_z = run_shape(cfg->path == OD_PATH_FUSED || cfg->path == OD_PATH_FUSED_GRAPH, &threads, &cpt);
+        p.threads = threads;
+        p.cpt = cpt;
+    }
 
     // tiles: full rows, balanced row slabs and plane chunks
     std::vector<int32_t> js, jl, ks, kl;
@@ -611,12 +639,20 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
         h.offRecv[1] = take(f_bytes);
     }
     p.arena_bytes = at;
-    if (!running && (run_z != tile_z || run_threads != p.threads)) {
-        // the arena also holds the tables of the tiles a context will run with
-        int64_t nt = 0, nd = 0;
-        count_tiles(p, (int64_t)run_threads * p.cpt, run_z, &nt, &nd);
-        const size_t mine = table_bytes((int64_t)p.tiles.size(), (int64_t)p.dep_idx.size()), run = table_bytes(nt, nd);
-        if (run > mine) p.arena_bytes += run - mine;
+    if (!running) {
+        // the arena also holds the tables of the tiles a context will run
+        // with, on any path
+        const size_t mine = table_bytes((int64_t)p.tiles.size(), (int64_t)p.dep_idx.size());
+        size_t most = mine;
+        for (int fused = 0; fused < 2; ++fused) {
+            int32_t threads, cpt;
+            const int32_t z = run_shape(fused != 0, &threads, &cpt);
+            if (z == tile_z && threads == p.threads && cpt == p.cpt) continue;
+            int64_t nt = 0, nd = 0;
+            count_tiles(p, (int64_t)threads * cpt, z, &nt, &nd);
+            most = std::max(most, table_bytes(nt, nd));
+        }
+        p.arena_bytes += most - mine;
     }
     return OD_OK;
 }
