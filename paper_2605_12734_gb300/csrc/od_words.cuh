@@ -28,9 +28,9 @@
 // producer that alternates strictly between issuing and finishing planes,
 // 0.541 event-driven, 0.524 with one 256-byte record per tile instead of five
 // dependent table reads, 0.489 with 6 ring slots (0.456 with the roundings left
-// out), 0.460 with rows of whole sectors (od_plan.cpp).  Two-dimensional,
-// 16384^2: 0.76 to 0.65.  What bounds it: at 32^3 chares the traffic (2.50 GB a
-// step, 0.80 of the copy bandwidth) and the ALU pipe (65 % busy, issue 71 %)
+// out), 0.460 with rows of whole sectors (od_plan.cpp), 0.443 with 256 x 4.  Two-dimensional,
+// 16384^2: 0.76 to 0.65.  What bounds it: at 32^3 chares the traffic (2.39 GB a
+// step, 0.79 of the copy bandwidth) and the ALU pipe (62 % busy, issue 67 %)
 // together; in two dimensions the copy bandwidth (0.99 of it).  A fused step on
 // the same case: 0.553 with a fixed stride of tiles per CTA, 0.480 by ticket.
 // Tried and slower: each thread's own cells of three planes kept in registers
