@@ -485,6 +485,10 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
                     __nanosleep(32);
                 }
             }
+            // Each lane has acquired the counters it watched, and a vote orders
+            // no memory: the barrier puts every lane's acquire before lane 0's
+            // copies and the other lanes' halo loads.
+            __syncwarp();
             // data written by other CTAs (generic proxy) is next read by bulk
             // copies (async proxy)
             asm volatile("fence.proxy.async.global;" ::: "memory");

@@ -1,0 +1,39 @@
+"""The producer warp of the sweep over fixed-point words on the GPU: what its
+lanes agree on before one of them acts for all, bit for bit against the CPU
+oracle."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def od():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2605_12734_gb300 import build
+    build.build()
+    import paper_2605_12734_gb300 as pkg
+    return pkg
+
+
+def same(got, want):
+    return np.array_equal(np.ascontiguousarray(got).view(np.uint64), np.ascontiguousarray(want).view(np.uint64))
+
+
+# every lane watches another tile's step counter (up to 19 in the tile's record,
+# more of them in the list), one plane or row to a tile, so that each step
+# hangs on tiles that other SMs finished just before
+@pytest.mark.parametrize("dims,kw", [
+    ((48, 40, 36), dict(split=(4, 5, 3), tile_y=2, tile_z=1)),
+    ((260, 128, 9), dict(cuts=([0, 4, 260], [0, 128], [0, 3, 9]))),
+    ((64, 64, 64), dict(split=(2, 2, 2), threads=256, cells_per_thread=1)),
+])
+def test_dependencies_watched_by_different_lanes(od, dims, kw):
+    want = oracle.solve(*dims, 11, 1, 150)
+    with od.Jacobi3D(*dims, seed=11, path="persistent", **kw) as s:
+        s.step(150)
+        assert same(s.read(), want)
