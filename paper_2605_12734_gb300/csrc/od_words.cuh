@@ -39,9 +39,11 @@
 // (+6000 cycles a tile), nanosleep in the producer's loop, taking the next
 // ticket earlier than the last plane's issue.
 //
-// Every wait is bounded.  Whoever runs into a limit records the error and
-// raises `stop`, which ends every other wait of the CTA; the producer leaves
-// last-issued copies in flight to no one: it waits, bounded, for them first.
+// Every wait is bounded, and no lane leaves its warp alone.  Whoever runs into
+// a limit on a phase raises `stop`, which ends every other such wait of the
+// CTA, and its warp records the error; a dependency wait that runs out records
+// the error and ends the CTA's tiles.  Copies in flight are left to no
+// one: the producer waits, bounded, for them before it leaves.
 #pragma once
 #include "od_plan.h"
 #include "od_tile.cuh"
@@ -94,22 +96,34 @@ struct WordsShared {
     uint32_t stop;
 };
 
-// Wait for a phase of `bar`; false when the limit ran out or the CTA stops.
-// The hardware suspends a try for a while by itself; the clock and the stop
-// word are looked at only between groups of tries, because reading the clock
-// takes longer than most waits.
-__device__ __forceinline__ bool wait_phase(uint64_t *bar, uint32_t parity, const uint32_t *stop, uint64_t limit_ns) {
-    if (mbar_try_wait(bar, parity)) return true;
+// Wait for a phase of `bar`, until it is there, the limit runs out or the CTA
+// stops.  The hardware suspends a try for a while by itself; the clock and the
+// stop word are looked at only between groups of tries, because reading the
+// clock takes longer than most waits.
+// A lane tries, reads the clock and reads the stop word for itself, so lanes of
+// one warp may differ in why they came back.  None acts on that alone: the one
+// that ran into the limit raises the stop word and goes on with its warp, which
+// asks `stopped` together before anything relies on the wait.
+__device__ __forceinline__ void wait_phase(uint64_t *bar, uint32_t parity, uint32_t *stop, uint64_t limit_ns) {
+    if (mbar_try_wait(bar, parity)) return;
     uint64_t t0 = 0;
     for (;;) {
 #pragma unroll 1
         for (int k = 0; k < 32; ++k)
-            if (mbar_try_wait(bar, parity)) return true;
-        if (*(const volatile uint32_t *)stop != 0u) return false;
+            if (mbar_try_wait(bar, parity)) return;
+        if (*(volatile uint32_t *)stop != 0u) return;
         const uint64_t t = now_ns();
         if (t0 == 0) t0 = t;
-        if (t - t0 > limit_ns) return false;
+        if (t - t0 > limit_ns) {
+            *(volatile uint32_t *)stop = 1u;
+            return;
+        }
     }
+}
+
+// Whether the CTA stops: one answer for a whole warp (all lanes together).
+__device__ __forceinline__ bool stopped(const uint32_t *stop) {
+    return __any_sync(0xFFFFFFFFu, *(const volatile uint32_t *)stop != 0u);
 }
 
 __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
@@ -294,8 +308,11 @@ __device__ __forceinline__ void words_compute(const KArgs &a, WordsShared &sh, c
     };
     for (uint32_t n = 0;; ++n) {
         const uint32_t i = n & 1u;
-        bool ok = wait_phase(&sh.told[i], (n >> 1) & 1u, &sh.stop, limit);
-        if (!ok) break;
+        wait_phase(&sh.told[i], (n >> 1) & 1u, &sh.stop, limit);
+        if (stopped(&sh.stop)) {
+            if (lane == 0) record_err(a.err, OD_ERR_TMA_TIMEOUT, -1, -1);  // (the first error stays)
+            break;
+        }
         const int tile = sh.t[i].tile;
         if (tile < 0) break;
         const int pitch = sh.t[i].pitch, plane = sh.t[i].plane;
@@ -319,16 +336,21 @@ __device__ __forceinline__ void words_compute(const KArgs &a, WordsShared &sh, c
         // the planes below the first computed one and that one
         uint64_t *held_d = &sh.empty[sl];  // the slots of planes k-1 and k
         const double *sd = ring + (size_t)sl * SD;
-        if (!wait_phase(&sh.ready[sl], ph, &sh.stop, limit)) break;
+        wait_phase(&sh.ready[sl], ph, &sh.stop, limit);
         advance();
         uint64_t *held_c = &sh.empty[sl];
         const double *sc = ring + (size_t)sl * SD;
-        if (!wait_phase(&sh.ready[sl], ph, &sh.stop, limit)) break;
+        wait_phase(&sh.ready[sl], ph, &sh.stop, limit);
         double *dpl = sh.t[i].dst;
-        for (int left = sh.t[i].nk; ok && left > 0; --left) {
+        // A warp whose wait ends without its phase goes on to the tile's end:
+        // it reads slots that may be half filled and stores into the tile's own
+        // cells of a context that has failed, and the tile is not published.
+        // (A vote on every wait instead: 512^3 in 32^3 chares 0.448 ms a step,
+        // 0.443 with this.)
+        for (int left = sh.t[i].nk; left > 0; --left) {
             advance();
             const double *su = ring + (size_t)sl * SD;
-            if (!(ok = wait_phase(&sh.ready[sl], ph, &sh.stop, limit))) break;
+            wait_phase(&sh.ready[sl], ph, &sh.stop, limit);
             // In the shapes of two cells a thread, which narrow planes get, a
             // warp past the plane's end has nothing to do and one in its last
             // part one cell (5195 x 7129 in 83-cell rows: 0.392 / 0.318 ms a
@@ -344,7 +366,10 @@ __device__ __forceinline__ void words_compute(const KArgs &a, WordsShared &sh, c
             sc = su;
             dpl += plane;
         }
-        if (!ok) break;
+        if (stopped(&sh.stop)) {
+            if (lane == 0) record_err(a.err, OD_ERR_TMA_TIMEOUT, tile, -1);
+            break;
+        }
         if (lane == 0) {
             mbar_arrive(held_d);
             mbar_arrive(held_c);
@@ -494,7 +519,8 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
             asm volatile("fence.proxy.async.global;" ::: "memory");
         }
         stage = 0;
-        if (n >= 2 && !wait_phase(&sh.taken[i], ((n >> 1) - 1u) & 1u, &sh.stop, 2u * a.spin_ns)) {
+        if (n >= 2) wait_phase(&sh.taken[i], ((n >> 1) - 1u) & 1u, &sh.stop, 2u * a.spin_ns);
+        if (stopped(&sh.stop)) {
             err = OD_ERR_TMA_TIMEOUT;
             break;
         }

@@ -37,3 +37,22 @@ def test_dependencies_watched_by_different_lanes(od, dims, kw):
     with od.Jacobi3D(*dims, seed=11, path="persistent", **kw) as s:
         s.step(150)
         assert same(s.read(), want)
+
+
+# a wait that runs out ends every warp of every CTA with the error recorded,
+# whatever the shape, and leaves the GPU to the next context
+@pytest.mark.parametrize("kw", [dict(threads=128, cells_per_thread=2), dict(threads=128, cells_per_thread=4),
+                                dict(threads=256, cells_per_thread=4), dict(threads=512, cells_per_thread=1)])
+@pytest.mark.parametrize("tile", [0, 5])
+def test_a_wait_that_runs_out_ends_the_launch(od, kw, tile):
+    with od.Jacobi3D(48, 40, 32, split=(2, 2, 2), seed=1, path="persistent", tile_z=4, spin_limit_ns=100_000_000,
+                     **kw) as s:
+        s.stall_tile(tile)
+        s.step(20)
+        with pytest.raises(od.ODError) as ei:
+            s.sync()
+        assert ei.value.status == od._native.OD_ETIMEOUT
+    want = oracle.solve(48, 40, 32, 1, 1, 20)
+    with od.Jacobi3D(48, 40, 32, split=(2, 2, 2), seed=1, path="persistent", tile_z=4, **kw) as s:
+        s.step(20)
+        assert same(s.read(), want)
