@@ -118,6 +118,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     }
 }
 
+// A CTA that gives up first lets its copies in flight land: one that lands
+// later would write into shared memory that another CTA has by then.  That wait
+// is bounded too, but by no less than a second, however short the limit that
+// ran out (od_config.spin_limit_ns).
+__device__ __forceinline__ uint64_t drain_limit(uint64_t limit_ns) {
+    return limit_ns > 1000000000ull ? limit_ns : 1000000000ull;
+}
+
 __device__ __forceinline__ void record_err(ErrDev *e, int code, int tile, int step) {
     if (atomicCAS(&e->code, 0, code) == 0) {
         e->tile = tile;
@@ -313,7 +321,8 @@ __device__ __forceinline__ bool run_tile(const KArgs &a, int tile_id, int sp, Ri
     // (a ring of S slots holds planes k-1, k, k+1 and S-3 planes in flight)
     auto drain = [&](int from) {
         if (tid == 0)
-            for (int p = from; p <= issued_hi; ++p) mbar_wait_bounded(ring.bars + slot(p), phase(p), g.spin_ns);
+            for (int p = from; p <= issued_hi; ++p)
+                mbar_wait_bounded(ring.bars + slot(p), phase(p), drain_limit(g.spin_ns));
         ring.seq = seq0 + (uint32_t)(issued_hi - kb + 1);
     };
 
@@ -572,7 +581,8 @@ __device__ __forceinline__ bool run_tile_2d(const KArgs &a, int tile_id, int sp,
     int issued_hi = kb - 1;
     auto drain = [&](int from) {
         if (tid == 0)
-            for (int p = from; p <= issued_hi; ++p) mbar_wait_bounded(ring.bars + slot(p), phase(p), g.spin_ns);
+            for (int p = from; p <= issued_hi; ++p)
+                mbar_wait_bounded(ring.bars + slot(p), phase(p), drain_limit(g.spin_ns));
         ring.seq = seq0 + (uint32_t)(issued_hi - kb + 1);
     };
 

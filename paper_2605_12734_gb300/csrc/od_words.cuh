@@ -673,7 +673,7 @@ __device__ __forceinline__ void words_produce(const KArgs &a, WordsShared &sh, d
         }
         // copies still in flight land before the CTA's shared memory is given up
         for (; in_flight > 0; --in_flight) {
-            mbar_wait_bounded(&sh.full[sf], pf, a.spin_ns);
+            mbar_wait_bounded(&sh.full[sf], pf, drain_limit(a.spin_ns));
             if (++sf == (uint32_t)S) {
                 sf = 0;
                 pf ^= 1u;

@@ -56,3 +56,23 @@ def test_a_wait_that_runs_out_ends_the_launch(od, kw, tile):
     with od.Jacobi3D(48, 40, 32, split=(2, 2, 2), seed=1, path="persistent", tile_z=4, **kw) as s:
         s.step(20)
         assert same(s.read(), want)
+
+
+# a wait limit too short for any copy: the launch ends with the error (or beats
+# the limit), its copies landed, and CTAs of other contexts, which take over the
+# shared memory, compute what they should
+@pytest.mark.parametrize("arith", [-1, 2])
+@pytest.mark.parametrize("path", ["persistent", "fused", "per_chare"])
+def test_copies_in_flight_land_before_a_cta_gives_up(od, path, arith):
+    dims = (256, 64, 48)
+    want = oracle.solve(*dims, 2, 1, 12)
+    with od.Jacobi3D(*dims, split=(2, 2, 2), seed=2, path=path, arith=arith) as good:
+        with od.Jacobi3D(*dims, split=(2, 2, 2), seed=2, path=path, arith=arith, spin_limit_ns=1) as s:
+            for _ in range(4):
+                good.step(3)
+                try:
+                    s.step(3)
+                    s.sync()
+                except od.ODError as e:
+                    assert e.status in (od._native.OD_ETIMEOUT, od._native.OD_ESTATE)
+        assert same(good.read(), want)
