@@ -895,7 +895,8 @@ od_status create_context(od_ctx **out, const od_config *cfg_in, bool sync) {
     od::Plan &p = c->plan;
     c->device = cfg->device;
     c->path = cfg->path;
-    c->spin_ns = cfg->spin_limit_ns ? cfg->spin_limit_ns : kDefaultSpinNs;
+    // (the sweep over words waits up to four times the limit: kept below 2^62)
+    c->spin_ns = std::min<uint64_t>(cfg->spin_limit_ns ? cfg->spin_limit_ns : kDefaultSpinNs, 1ull << 61);
     DeviceGuard dg(c->device);
     if (!dg.ok) {
         release(c);

@@ -76,3 +76,12 @@ def test_copies_in_flight_land_before_a_cta_gives_up(od, path, arith):
                 except od.ODError as e:
                     assert e.status in (od._native.OD_ETIMEOUT, od._native.OD_ESTATE)
         assert same(good.read(), want)
+
+
+# limits as good as none, whose multiples by 2 and 4 pass the end of 64 bits
+@pytest.mark.parametrize("limit", [1 << 61, 1 << 62, (1 << 62) + 1, 1 << 63, (1 << 64) - 1])
+def test_wait_limits_of_any_size(od, limit):
+    want = oracle.solve(64, 64, 64, 7, 1, 40)
+    with od.Jacobi3D(64, 64, 64, split=(2, 2, 2), seed=7, path="persistent", spin_limit_ns=limit) as s:
+        s.step(40)
+        assert same(s.read(), want)
