@@ -1125,6 +1125,9 @@ od_status od_read(od_ctx *c, double *dst, int32_t dst_is_device) {
     // the export follows the steps on the stream, and one wait at the end
     // covers both and the error record
     if (dst_is_device || mapped) {
+        // a pending od_read_async may still be filling the same buffer from its
+        // copy stream (the staging branch waits for it in ensure_stage)
+        if (c->copy_pending) OD_CUDA(cudaStreamWaitEvent(c->stream, c->ev_copied, 0));
         e = od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, dst_is_device ? dst : mapped, c->d_fmt,
                               c->stream);
     } else {
