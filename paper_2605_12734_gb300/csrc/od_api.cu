@@ -1120,26 +1120,27 @@ od_status od_read(od_ctx *c, double *dst, int32_t dst_is_device) {
     const od::Plan &p = c->plan;
     const int par = (int)(c->steps & 1);
     double *mapped = dst_is_device ? nullptr : device_view(dst);
-    od_status s = OD_OK;
-    cudaError_t e = cudaSuccess;
-    // the export follows the steps on the stream, and one wait at the end
-    // covers both and the error record
     if (dst_is_device || mapped) {
         // a pending od_read_async may still be filling the same buffer from its
         // copy stream (the staging branch waits for it in ensure_stage)
         if (c->copy_pending) OD_CUDA(cudaStreamWaitEvent(c->stream, c->ev_copied, 0));
-        e = od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, dst_is_device ? dst : mapped, c->d_fmt,
-                              c->stream);
-    } else {
-        s = ensure_stage(c);
-        if (s != OD_OK) return s;
-        e = od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, c->d_stage, c->d_fmt, c->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(dst, c->d_stage, (size_t)p.cells * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+        // the export follows the steps on the stream, and one wait at the end
+        // covers both and the error record; it does nothing if a step failed
+        const cudaError_t e = od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny,
+                                                dst_is_device ? dst : mapped, c->d_fmt, c->d_err, c->stream);
+        const od_status s = check_device_error_impl(c);
+        return s == OD_OK && e != cudaSuccess ? cuda_fail(e, "od_read") : s;
     }
+    od_status s = ensure_stage(c);
+    if (s != OD_OK) return s;
+    const cudaError_t e = od::launch_gather(c->d_ch, (int)p.ch.size(), par, p.nx, p.ny, c->d_stage, c->d_fmt, nullptr,
+                                            c->stream);
     s = check_device_error_impl(c);
-    if (s == OD_OK && e != cudaSuccess) s = cuda_fail(e, "od_read");
-    return s;
+    if (s != OD_OK) return s;
+    if (e != cudaSuccess) return cuda_fail(e, "od_read");
+    OD_CUDA(cudaMemcpyAsync(dst, c->d_stage, (size_t)p.cells * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    OD_CUDA(cudaStreamSynchronize(c->stream));
+    return OD_OK;
 }
 
 od_status od_write(od_ctx *c, const double *src, int32_t src_is_device) {
@@ -1194,7 +1195,8 @@ od_status od_read_async(od_ctx *c, double *dst) {
         OD_CUDA(cudaEventCreateWithFlags(&c->ev_copied, cudaEventDisableTiming));
     }
     const od::Plan &p = c->plan;
-    OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), (int)(c->steps & 1), p.nx, p.ny, c->d_stage, c->d_fmt, c->stream));
+    OD_CUDA(od::launch_gather(c->d_ch, (int)p.ch.size(), (int)(c->steps & 1), p.nx, p.ny, c->d_stage, c->d_fmt, nullptr,
+                              c->stream));
     OD_CUDA(cudaEventRecord(c->ev_gathered, c->stream));
     OD_CUDA(cudaStreamWaitEvent(c->copy_stream, c->ev_gathered, 0));
     OD_CUDA(cudaMemcpyAsync(dst, c->d_stage, (size_t)p.cells * sizeof(double), cudaMemcpyDeviceToHost,

@@ -319,7 +319,11 @@ constexpr int kIoRows = 4;
 // A11: interiors of parity p -> global x-fastest array.  Each warp moves
 // kIoRows interior rows per pass (coalesced on both sides), one 32-bit
 // division per row.
-__global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, double *g, const FmtDev *fmt) {
+// err (may be null): a launch before this one that gave up has left no field
+// to export, and g stays as it is.
+__global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, double *g, const FmtDev *fmt,
+                         const ErrDev *err) {
+    if (err && err->code != 0) return;
     const uint32_t base = fmt->base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int c = blockIdx.y; c < nch; c += gridDim.y) {
@@ -633,8 +637,8 @@ cudaError_t launch_read_cells(const double *const *addr, int64_t n, double *out,
 }
 
 cudaError_t launch_gather(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, double *g,
-                          const FmtDev *fmt, cudaStream_t s) {
-    k_gather<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, parity, nx, ny, g, fmt);
+                          const FmtDev *fmt, const ErrDev *err, cudaStream_t s) {
+    k_gather<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, parity, nx, ny, g, fmt, err);
     return cudaGetLastError();
 }
 

@@ -69,8 +69,9 @@ cudaError_t launch_pack(const ChareDev *ch, int c, int parity, int elems, cudaSt
 cudaError_t launch_unpack(const ChareDev *ch, int c, int parity, int slot, int elems, cudaStream_t s);
 // out[i] = *addr[i] for n device addresses (od_read_cells).
 cudaError_t launch_read_cells(const double *const *addr, int64_t n, double *out, const FmtDev *fmt, cudaStream_t s);
+// Export; with err (device record, may be null) only if no launch before it failed.
 cudaError_t launch_gather(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, double *g,
-                          const FmtDev *fmt, cudaStream_t s);
+                          const FmtDev *fmt, const ErrDev *err, cudaStream_t s);
 // Arithmetic self-test over device arrays (op: 0 div6, 1 add on the integer
 // pipes; 2 division by 6, 3 add on the FP64 pipe).
 cudaError_t launch_arith(int op, const double *a, const double *b, double *out, int64_t n, cudaStream_t s);

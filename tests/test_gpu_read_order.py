@@ -43,3 +43,24 @@ def test_read_into_the_buffer_of_a_pending_export(od, how):
         s.sync()
         assert same(first, want)
         assert same(buf.numpy(), want)
+
+
+# a read that reports the error of a launch that gave up leaves dst alone
+@pytest.mark.parametrize("where", ["device", "pinned", "pageable"])
+@pytest.mark.parametrize("arith", [-1, 12, 2])
+def test_read_of_a_failed_context_leaves_dst(od, where, arith):
+    import torch
+    n = 48
+    if where == "device":
+        dst = torch.full((n ** 3,), -3.0, dtype=torch.float64, device="cuda:0")
+    else:
+        dst = torch.full((n ** 3,), -3.0, dtype=torch.float64, pin_memory=where == "pinned").numpy()
+    with od.Jacobi3D(n, n, n, split=(2, 2, 2), seed=1, path="persistent", arith=arith,
+                     spin_limit_ns=100_000_000) as s:
+        s.stall_tile(0)
+        s.step(3)
+        for _ in range(2):
+            with pytest.raises(od.ODError) as ei:
+                s.read(dst)
+            assert ei.value.status == od._native.OD_ETIMEOUT
+            assert bool((dst == -3.0).all())
