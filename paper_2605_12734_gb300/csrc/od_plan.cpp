@@ -59,6 +59,9 @@ bool edges_from(int64_t n, int32_t p, const int32_t *cuts, int32_t ncuts, const 
     return true;
 }
 
+// doubles from one row of a chare to the next (see ChareDev)
+int32_t row_pitch(int32_t bx) { return bx % 4 == 0 ? bx + 4 : round_up(bx + 2, 2); }
+
 // split n into parts of at most `cap`, balanced
 void balanced_parts(int32_t n, int32_t cap, std::vector<int32_t> *starts, std::vector<int32_t> *lens) {
     int32_t parts = (n + cap - 1) / cap;
@@ -139,6 +142,20 @@ static size_t table_bytes(int64_t nt, int64_t nd) {
            a((size_t)std::max<int64_t>(1, nd) * 4) + a((size_t)nt * 4) + a((size_t)nt * sizeof(TileRec));
 }
 
+// A ring of `stages` slots (0: of the planner's choice, 4 at least) for the wider
+// tiles has to fit beside the kernel's own shared memory; it may not only for
+// rows of a few cells in a ring of 7 or 8 slots.
+static bool words_ring_fits(const Plan &p, int32_t stages, int32_t threads, int32_t cpt) {
+    int64_t slot = 0;
+    for (size_t a = 1; a < p.ex.size(); ++a)
+        for (size_t b = 1; b < p.ey.size(); ++b) {
+            const int32_t w = (int32_t)(p.ex[a] - p.ex[a - 1]), h = (int32_t)(p.ey[b] - p.ey[b - 1]);
+            const int32_t rows = std::min(h, threads * cpt / w), parts = (h + rows - 1) / rows;
+            slot = std::max<int64_t>(slot, stage_doubles_for((h + parts - 1) / parts, row_pitch(w)));
+        }
+    return kSmemHeader + (stages ? stages : 4) * slot * 8 + words_static_smem(threads) <= kMaxSmem;
+}
+
 // Threads and cells a thread with which a context's sweep over words runs where
 // the plan, not told a shape, reports 128 x 2 or 128 x 4 (cells a CTA: 256, 512).
 // A CTA of twice the cells has tiles of twice the rows: half the halo rows
@@ -158,7 +175,7 @@ static size_t table_bytes(int64_t nt, int64_t nd) {
 // 24^3 chares fill 9/16: 663 / 634, but a fused step 639 / 658.  Grids under
 // 2^19 cells keep the reported shape (64^3 in 8 chares: 7.6 / 7.8 / 7.4, fused
 // 9.2 / 9.7 / 10.3).
-static void words_shape(const Plan &p, bool fused, int32_t *threads, int32_t *cpt) {
+static void words_shape(const Plan &p, bool fused, int32_t stages, int32_t *threads, int32_t *cpt) {
     if (p.stencil != OD_STENCIL_3D7 || p.threads != 128 || (p.cpt != 2 && p.cpt != 4) || p.tile_y > 0 ||
         p.nx * p.ny * p.nz < (1 << 19))
         return;
@@ -171,8 +188,10 @@ static void words_shape(const Plan &p, bool fused, int32_t *threads, int32_t *cp
             }
         return n;
     };
-    if (*cpt == 2 && lanes(512) <= lanes(256)) *cpt = 4;
-    if (*cpt != 4 || lanes(1024) > lanes(512) || p.nx * p.ny * 8 < lanes(1024) * 5) return;
+    if (*cpt == 2 && lanes(512) <= lanes(256) && words_ring_fits(p, stages, 128, 4)) *cpt = 4;
+    if (*cpt != 4 || lanes(1024) > lanes(512) || p.nx * p.ny * 8 < lanes(1024) * 5 ||
+        !words_ring_fits(p, stages, 256, 4))
+        return;
     int64_t nt = 0, nd = 0;
     if (fused) count_tiles(p, 1024, 32, &nt, &nd);
     if (!fused || nt >= 3 * 3 * 152) *threads = 256;  // three resident CTAs an SM
@@ -396,7 +415,7 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
                 h.y0 = p.ey[cy]; h.by = (int32_t)(p.ey[cy + 1] - p.ey[cy]);
                 h.z0 = p.ez[cz]; h.bz = (int32_t)(p.ez[cz + 1] - p.ez[cz]);
                 h.col0 = h.bx % 4 == 0 ? 4 : 1;
-                h.pitch = h.bx % 4 == 0 ? h.bx + 4 : round_up(h.bx + 2, 2);
+                h.pitch = row_pitch(h.bx);
                 h.rows = p.stencil == OD_STENCIL_2D5 ? 1 : h.by + 2;
                 h.row0 = p.stencil == OD_STENCIL_2D5 ? 0 : 1;
                 h.nbr[OD_FACE_XLO] = cx > 0 ? (int32_t)(c - 1) : -1;
@@ -429,7 +448,7 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     auto run_shape = [&](bool fused, int32_t *threads, int32_t *cpt) {  // returns the planes per tile
         *threads = p.threads;
         *cpt = p.cpt;
-        if (words && auto_shape && fill_gpu) words_shape(p, fused, threads, cpt);
+        if (words && auto_shape && fill_gpu) words_shape(p, fused, cfg->stages, threads, cpt);
         return cfg->tile_z > 0 ? cfg->tile_z : words ? words_tile_z(p, *threads, *cpt) : 32;
     };
     int32_t tile_z = cfg->tile_z > 0 ? cfg->tile_z : 32;

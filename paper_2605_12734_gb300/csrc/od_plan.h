@@ -25,6 +25,9 @@ constexpr int words_regs(int cpt, bool d3) { return cpt > 4 ? 112 : d3 ? 64 : 56
 constexpr int words_ctas(int nt, int cpt, bool d3) {
     return 65536 / (words_regs(cpt, d3) * (nt + 32)) > 1 ? 65536 / (words_regs(cpt, d3) * (nt + 32)) : 1;
 }
+// Their static shared memory: barriers, tile records and counters (WordsShared),
+// and from 256 compute threads on the lists of words_redo.
+constexpr int words_static_smem(int nt) { return 1280 + (nt >= 256 ? 2048 : 0); }
 inline int32_t kernel_mode(int32_t arith, bool words) { return words && arith == kDefaultArith ? kFxMode : arith; }
 
 struct HostChare {

@@ -95,6 +95,7 @@ struct WordsShared {
     TileRec rec[2];      // the producer's: its tile's record and the next one's
     uint32_t stop;
 };
+static_assert(sizeof(WordsShared) <= words_static_smem(128), "the planner's figure for it");
 
 // Wait for a phase of `bar`, until it is there, the limit runs out or the CTA
 // stops.  The hardware suspends a try for a while by itself; the clock and the
@@ -159,6 +160,9 @@ __device__ __forceinline__ uint32_t count_acq_rel(uint32_t *p) {
 // from a uniform random field, 2 % of the cells, 512^3 in 64^3 chares: 1.31 ms
 // without, 1.07 with it; 40 steps from a cold 200^3 field 3.88 and 3.48).
 // Out of line: 64^3 chares in 256 x 4 0.427 ms a step, inlined 0.433.
+constexpr int kRedoWarps = 16;  // of a CTA of up to 512 compute threads
+static_assert(kRedoWarps * 32 * 4 <= words_static_smem(256) - words_static_smem(128), "the planner's figure for it");
+
 template <int N>
 struct Offsets {
     int r[N];
@@ -168,7 +172,7 @@ template <int ST, int N>
 static __device__ __noinline__ void words_redo(const double *sd, const double *sc, const double *su, double *dpl,
                                                Offsets<N> rf, int pitch, uint32_t e0, bool rare) {
     constexpr bool k3D = ST == OD_STENCIL_3D7;
-    __shared__ int32_t lists[16][32];  // one per warp of a CTA of up to 512 compute threads
+    __shared__ int32_t lists[kRedoWarps][32];
     int32_t *list = lists[threadIdx.x >> 5];
     const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
     uint32_t number[N], total = 0;

@@ -167,3 +167,13 @@ def test_allocation_free_entry(od, dims, kind):
         shell = np.ones(P.shape, dtype=bool)
         shell[1:-1, 1:-1, 1:-1] = False
         assert same(got[shell], P[shell])  # carried over unchanged
+
+
+# rows of one cell in a ring too deep for the wider tiles
+@pytest.mark.parametrize("path", ["persistent", "fused", "per_chare"])
+@pytest.mark.parametrize("stages", [7, 8])
+def test_deep_rings_of_narrow_rows(od, path, stages):
+    want = oracle.solve(1, 2048, 512, 2, 1, 3)
+    with od.Jacobi3D(1, 2048, 512, split=(1, 1, 1), seed=2, path=path, stages=stages) as s:
+        s.step(3)
+        assert same(s.read(), want)
