@@ -17,6 +17,8 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int32_t kMaxSmem = 232448;  // 227 KB opt-in per CTA on sm_100/sm_103
+constexpr int32_t kSmemPerSM = 233472;  // 228 KB
+constexpr int32_t kSmemReserved = 1024;  // of it, kept by the hardware for each resident CTA
 constexpr int32_t kSmemHeader = 256;  // mbarriers + neighbour push table
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -539,10 +541,13 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     // memory of the CTAs that the registers admit, up to 6 planes (3D; 0.524 ms
     // a step with 4, 0.500 with 5, 0.489 with 6 at 512^3 in 4096 chares) or 8
     // rows (2D; 16384^2 0.745 ms with 4, 0.665 with 8); never fewer than the 4
-    // of the other sweeps.
+    // of the other sweeps.  One slot more than fits costs a resident CTA: 256-cell
+    // rows (256 x 4), 512^3 in 8 chares with 6 slots and 2 CTAs an SM 0.476 ms a
+    // step, with 5 and 3 0.432; 460-cell rows with 5 and 2 0.383, 4 and 3 0.369.
     if (cfg->stages == 0 && p.amode == kDefaultArith) {
         const bool d3 = p.stencil == OD_STENCIL_3D7;
-        const int64_t per_cta = 228 * 1024 / words_ctas(p.threads, p.cpt, d3) - 2048 - kSmemHeader;
+        const int64_t per_cta = kSmemPerSM / words_ctas(p.threads, p.cpt, d3) - kSmemReserved -
+                                words_static_smem(p.threads) - kSmemHeader;
         const int64_t fit = per_cta / ((int64_t)p.stage_doubles * 8);
         p.stages = (int32_t)std::max<int64_t>(4, std::min<int64_t>(d3 ? 6 : 8, fit));
     }

@@ -77,3 +77,17 @@ def test_what_is_reported_is_accepted(running):
         stages, path = rng.choice([0, 3, 5, 7, 8]), rng.randint(0, 4)
         if running(dims, split, path=path, stages=stages, run=False):
             assert running(dims, split, path=path, stages=stages), (dims, split, stages, path)
+
+
+# the ring is as deep as it can be without taking a CTA's place on the SM
+@pytest.mark.parametrize("stencil", [0, 1])
+def test_ring_depth_leaves_room_for_the_resident_ctas(running, stencil):
+    deep = 0
+    for width in range(4, 1200, 3):
+        dims, split = ((width, 260, 260), (1, 1, 1)) if stencil == 0 else ((width * 4, 900, 1), (4, 3, 1))
+        for path in (1, 3):
+            p = running(dims, split, stencil=stencil, path=path)
+            if p["stages"] > 4:
+                deep += 1
+                assert p["ctas"] * (p["smem"] + p["static_smem"] + RESERVED) <= PER_SM, (width, path, p)
+    assert deep > 300
