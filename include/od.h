@@ -165,8 +165,8 @@ typedef struct od_config {
                                     other / every fourth cell, 12 on the rest.
                                     Mode 12 keeps the field itself as words of
                                     such a window where it can (from od_create
-                                    or od_write on; until a face is imported or
-                                    a field reaches 2^757) and then needs no
+                                    or od_write on; until the field or a face
+                                    fed to it reaches 2^757) and then needs no
                                     FP64 add.
                                     2D: 12 one FP64 add and two window adds,
                                     13 none and three, 14 the two mixed, 15
@@ -316,7 +316,8 @@ OD_API od_status od_read_cells(od_ctx *ctx, const int64_t *cells, int64_t n, dou
  * Dirichlet shell is kept.  Used to import a checkpoint or a user field.
  * Enqueued on the stream (host sources are copied before return).  The
  * context keeps the largest positive value its field has held (the initial
- * field's values lie in [0, 1)), raised here by the values written; the
+ * field's values lie in [0, 1)), raised here by the values written (and, in
+ * the default arithmetic, by the faces that od_face_copy imports); the
  * anchored arithmetic modes place their integer window there, so a field
  * that later lies far below that value runs mostly in the IEEE form --
  * slower, with the same bits. */

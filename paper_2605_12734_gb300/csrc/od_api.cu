@@ -478,19 +478,10 @@ od_status ensure_stage(od_ctx *c) {
     return OD_OK;
 }
 
-// The captured step loops (they are captured again when next needed).
-void drop_graphs(od_ctx *c) {
-    for (cudaGraphExec_t *g : {&c->g2, &c->g1[0], &c->g1[1], &c->gf, &c->gf1[0], &c->gf1[1]}) {
-        if (*g) cudaGraphExecDestroy(*g);
-        *g = nullptr;
-    }
-    c->g2_kernels = c->g1_kernels[0] = c->g1_kernels[1] = 0;
-    c->g2_calls = c->g1_calls[0] = c->g1_calls[1] = 0;
-}
-
 void release(od_ctx *c) {
     if (!c) return;
-    drop_graphs(c);
+    for (cudaGraphExec_t g : {c->g2, c->g1[0], c->g1[1], c->gf, c->gf1[0], c->gf1[1]})
+        if (g) cudaGraphExecDestroy(g);
     for (auto e : c->ev) cudaEventDestroy(e);
     for (auto e : c->join) cudaEventDestroy(e);
     if (c->fork) cudaEventDestroy(c->fork);
@@ -502,6 +493,7 @@ void release(od_ctx *c) {
     if (c->ev_gathered) cudaEventDestroy(c->ev_gathered);
     if (c->ev_copied) cudaEventDestroy(c->ev_copied);
     if (c->d_stage) cudaFree(c->d_stage);
+    if (c->wider) cudaFreeHost(c->wider);
     if (c->own_arena && c->arena) cudaFree(c->arena);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -1034,6 +1026,13 @@ od_status od_step(od_ctx *c, int32_t iters) {
     if (c->failed) return fail(OD_ESTATE, "context failed earlier; destroy it");
     if (iters == 0) return OD_OK;
     DeviceGuard dg(c->device);
+    // a face import asked for a wider format (or will, when its kernel has run:
+    // until then the cells beside the larger values are only slower)
+    if (c->wider && *(volatile uint32_t *)c->wider != 0u) {
+        *(volatile uint32_t *)c->wider = 0u;
+        OD_CUDA(od::launch_refit(c->d_ch, (int)c->plan.ch.size(), (int)(c->steps & 1), c->plan.nx, c->plan.ny,
+                                 c->d_vmax, c->d_fmt, c->stream));
+    }
     switch (c->path) {
         case OD_PATH_FUSED:
         case OD_PATH_FUSED_GRAPH:
@@ -1220,20 +1219,21 @@ od_status od_face_copy(od_ctx *c, int32_t face, int32_t dir, double *buf, int32_
     const int64_t n = f < 2 ? p.ny * p.nz : f < 4 ? p.nx * p.nz : p.nx * p.ny;
     DeviceGuard dg(c->device);
     const int par = (int)(c->steps & 1);
-    const int nch = (int)p.ch.size();
-    if (dir == 1 && c->words) {
-        // values from outside may exceed the field's own largest, which its
-        // words rely on: from here on the context holds plain doubles
-        OD_CUDA(od::launch_plain(c->d_ch, nch, c->d_fmt, c->stream));
-        c->words = false;
-        drop_graphs(c);  // captured with the kernels over words
+    if (dir == 1 && c->words && !c->wider) {  // the first import
+        OD_CUDA(cudaHostAlloc(&c->wider, sizeof *c->wider, cudaHostAllocMapped));
+        *c->wider = 0u;
     }
+    // the copy between the device-visible buffer b and the field
+    auto copy = [&](double *b) {
+        return od::launch_face_copy(c->d_ch, p.px, p.py, p.pz, par, f, dir, b, p.nx, p.ny, p.nz,
+                                    c->words ? c->d_vmax : nullptr, c->d_fmt, c->wider, c->stream);
+    };
     if (buf_is_device) {
-        OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, buf, p.nx, p.ny, p.nz, c->d_fmt, c->stream));
+        OD_CUDA(copy(buf));
         return OD_OK;
     }
     if (double *mapped = device_view(buf)) {  // pinned host memory: in place
-        OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, mapped, p.nx, p.ny, p.nz, c->d_fmt, c->stream));
+        OD_CUDA(copy(mapped));
         OD_CUDA(cudaStreamSynchronize(c->stream));
         return OD_OK;
     }
@@ -1241,7 +1241,7 @@ od_status od_face_copy(od_ctx *c, int32_t face, int32_t dir, double *buf, int32_
     if (s != OD_OK) return s;
     if (dir == 1)
         OD_CUDA(cudaMemcpyAsync(c->d_stage, buf, (size_t)n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    OD_CUDA(od::launch_face_copy(c->d_ch, nch, par, f, dir, c->d_stage, p.nx, p.ny, p.nz, c->d_fmt, c->stream));
+    OD_CUDA(copy(c->d_stage));
     if (dir == 0)
         OD_CUDA(cudaMemcpyAsync(buf, c->d_stage, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     OD_CUDA(cudaStreamSynchronize(c->stream));

@@ -30,7 +30,8 @@ struct od_ctx {
     uint64_t *d_vmax = nullptr;       // largest value of the field (bits), in the arena's queue block
     FmtDev *d_fmt = nullptr;          // format of the field's words, beside it
     bool words = false;               // the field may be kept as fixed-point words (the default
-                                      // arithmetic, until a face is fed from outside)
+                                      // arithmetic, if the ring leaves its kernels room)
+    uint32_t *wider = nullptr;        // mapped host word: a face import asks for another format
     bool ghosts_current = true;       // internal ghost layers of the current parity hold the
                                       // neighbours' faces (false after a fused step or an import)
     std::vector<ChareDev> h_ch;       // host copy (device pointers)

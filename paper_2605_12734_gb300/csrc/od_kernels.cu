@@ -274,33 +274,92 @@ __global__ void k_ghost_refresh(const ChareDev *ch, int nch, int p) {
     }
 }
 
-// Domain-face exchange of a shard: the chares on domain face f (no neighbour
-// there) copy, cell by cell, their boundary layer of parity p into buf
-// (dir 0) or buf into their ghost layer (dir 1).  buf is the whole face,
-// dense: x faces nz x ny (y fastest), y faces nz x nx, z faces ny x nx (x
-// fastest).
-__global__ void k_face_copy(const ChareDev *ch, int nch, int p, int f, int dir, double *buf, int64_t nx, int64_t ny,
-                            int64_t nz, const FmtDev *fmt) {
-    const uint32_t base = fmt->base;
-    for (int c = blockIdx.y; c < nch; c += gridDim.y) {
+// Every word of both parities to plain doubles, by one block.
+__device__ void whole_to_plain(const ChareDev *ch, int nch, uint32_t base) {
+    for (int c = 0; c < nch; ++c) {
         const ChareDev &C = ch[c];
-        const bool on_face = f == OD_FACE_XLO ? C.x0 == 0 : f == OD_FACE_XHI ? C.x0 + C.bx == nx
-                           : f == OD_FACE_YLO ? C.y0 == 0 : f == OD_FACE_YHI ? C.y0 + C.by == ny
-                           : f == OD_FACE_ZLO ? C.z0 == 0 : C.z0 + C.bz == nz;
-        if (!on_face) continue;
-        const int n = f < 2 ? C.by * C.bz : f < 4 ? C.bx * C.bz : C.bx * C.by;
-        const int w = f < 2 ? C.by : C.bx;  // fastest extent of the chare's face
-        for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-            const int a = q % w, b = q / w;
-            int64_t g;  // position in buf
-            if (f < 2) g = (C.z0 + b) * ny + C.y0 + a;
-            else if (f < 4) g = (C.z0 + b) * nx + C.x0 + a;
-            else g = (C.y0 + b) * nx + C.x0 + a;
-            const int64_t o = face_offset(C, f, q, dir != 0);
-            if (dir == 0) buf[g] = fx_decode(f64_bits(C.A[p][o]), base);
-            else C.A[p][o] = f64_from(fx_encode(buf[g], base));
+        const int64_t n = (int64_t)C.rows * (C.bz + 2) * C.pitch;
+        for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
+            C.A[0][e] = fx_decode(f64_bits(C.A[0][e]), base);
+            C.A[1][e] = fx_decode(f64_bits(C.A[1][e]), base);
         }
     }
+}
+
+// Domain-face exchange of a shard: the chares on domain face f (no neighbour
+// there; chare first + a * step_a + b * step_b is its a-th and b-th, na x nb of
+// them) copy, cell by cell, their boundary layer of parity p into buf (dir 0)
+// or buf into their ghost layer (dir 1).  buf is the whole face, dense: x faces
+// nz x ny (y fastest), y faces nz x nx, z faces ny x nx (x fastest).
+//
+// An import (vmax not null: of a context that may hold words) also raises *vmax
+// to the face's largest positive finite value, on which the words rely.  A
+// value above their window but below 2^757 has a word all the same, and only
+// the cells beside it are slower: *wider (mapped host memory) then asks the
+// host to refit the field before a later step.  A larger one would not: the
+// last block to finish turns the whole context to plain doubles, alone and
+// slowly, once in a context's life, and writes the face again.
+struct FaceChares {
+    int32_t first, step_a, na, step_b, nb;
+};
+
+__global__ void k_face_copy(const ChareDev *ch, int nch, FaceChares on, int p, int f, int dir, double *buf, int64_t nx,
+                            int64_t ny, int64_t nz, unsigned long long *vmax, FmtDev *fmt, uint32_t *wider) {
+    const uint32_t base = fmt->base;
+    unsigned long long vm = 0;
+    auto copy = [&](int s0, int sn, int t0, int tn, uint32_t e0) {
+        for (int s = s0; s < on.na * on.nb; s += sn) {
+            const int sb = s / on.na, sa = s - sb * on.na;
+            const ChareDev &C = ch[on.first + sa * on.step_a + sb * on.step_b];
+            const int n = f < 2 ? C.by * C.bz : f < 4 ? C.bx * C.bz : C.bx * C.by;
+            const int w = f < 2 ? C.by : C.bx;  // fastest extent of the chare's face
+            for (int q = t0; q < n; q += tn) {
+                const int b = q / w, a = q - b * w;
+                int64_t g;  // position in buf
+                if (f < 2) g = (C.z0 + b) * ny + C.y0 + a;
+                else if (f < 4) g = (C.z0 + b) * nx + C.x0 + a;
+                else g = (C.y0 + b) * nx + C.x0 + a;
+                const int64_t o = face_offset(C, f, q, dir != 0);
+                if (dir == 0) {
+                    buf[g] = fx_decode(f64_bits(C.A[p][o]), e0);
+                } else {
+                    const double v = buf[g];
+                    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+                    if (bits < 0x7FF0000000000000ull && bits > vm) vm = bits;  // positive and finite
+                    C.A[p][o] = f64_from(fx_encode(v, e0));
+                }
+            }
+        }
+    };
+    copy(blockIdx.y, gridDim.y, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, base);
+    if (dir == 0 || !vmax) return;
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = __shfl_xor_sync(0xFFFFFFFFu, vm, o);
+        if (w > vm) vm = w;
+    }
+    if ((threadIdx.x & 31) == 0 && vm > *(volatile unsigned long long *)vmax) atomicMax(vmax, vm);
+    if (base == 0u) return;
+    __shared__ uint32_t s_to;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_to = base;
+        if (atomicAdd(&fmt->done, 1u) == gridDim.x * gridDim.y - 1u) {  // the last block: *vmax is the field's
+            fmt->done = 0u;
+            __threadfence();
+            s_to = fx_anchor(*(volatile unsigned long long *)vmax);
+        }
+    }
+    __syncthreads();
+    if (s_to == base) return;
+    if (s_to != 0u) {
+        if (threadIdx.x == 0) *(volatile uint32_t *)wider = 1u;
+        return;
+    }
+    whole_to_plain(ch, nch, base);
+    __syncthreads();
+    copy(0, 1, threadIdx.x, blockDim.x, 0u);
+    if (threadIdx.x == 0) fmt->base = 0u;
 }
 
 // Selected cells: out[i] = the value at *addr[i] (addresses inside the chares' arrays).
@@ -408,11 +467,12 @@ __global__ void k_scatter(const ChareDev *ch, int nch, int p, int64_t nx, int64_
 // After an import: the field's largest value may have outgrown the format it
 // was written in.  If it has (every block finds the same answer: nothing else
 // writes these words), the whole field takes the format that its largest
-// value asks for: the interiors of parity p from the import's source again,
-// every ghost cell of both parities (the Dirichlet shell among them) from its
-// present words; the other parity's interiors are written before they are
-// read.  The last block records the format.  A field that stayed within its
-// format costs one launch that reads two words.
+// value asks for: the interiors of parity p from the import's source again (g;
+// null: from their present words, after a face's import), every ghost cell of
+// both parities (the Dirichlet shell among them) from its present words; the
+// other parity's interiors are written before they are read.  The last block
+// records the format.  A field that stayed within its format costs one launch
+// that reads two words.
 __global__ void k_refit(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, const double *g,
                         const unsigned long long *vmax, FmtDev *fmt) {
     const uint32_t from = fmt->base;
@@ -431,7 +491,9 @@ __global__ void k_refit(const ChareDev *ch, int nch, int p, int64_t nx, int64_t 
             double *a = C.A[p] + (int64_t)rr * C.pitch, *b = C.A[p ^ 1] + (int64_t)rr * C.pitch;
             for (int cp = lane; cp < C.pitch; cp += 32) {
                 if (inside && cp >= C.col0 && cp < C.col0 + C.bx) {
-                    a[cp] = f64_from(fx_encode(g[((C.z0 + k) * ny + C.y0 + j) * nx + C.x0 + cp - C.col0], to));
+                    const double v = g ? g[((C.z0 + k) * ny + C.y0 + j) * nx + C.x0 + cp - C.col0]
+                                       : fx_decode(f64_bits(a[cp]), from);
+                    a[cp] = f64_from(fx_encode(v, to));
                 } else {
                     a[cp] = f64_from(fx_encode(fx_decode(f64_bits(a[cp]), from), to));
                     b[cp] = f64_from(fx_encode(fx_decode(f64_bits(b[cp]), from), to));
@@ -445,21 +507,6 @@ __global__ void k_refit(const ChareDev *ch, int nch, int p, int64_t nx, int64_t 
         if (atomicAdd(&fmt->done, 1u) == gridDim.x - 1u) {
             fmt->done = 0u;
             fmt->base = to;
-        }
-    }
-}
-
-// Every word of both parities to plain doubles (the caller clears the format
-// word behind it).
-__global__ void k_plain(const ChareDev *ch, int nch, const FmtDev *fmt) {
-    const uint32_t base = fmt->base;
-    if (base == 0u) return;
-    for (int c = blockIdx.y; c < nch; c += gridDim.y) {
-        const ChareDev &C = ch[c];
-        const int64_t n = (int64_t)C.rows * (C.bz + 2) * C.pitch;
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-            C.A[0][e] = fx_decode(f64_bits(C.A[0][e]), base);
-            C.A[1][e] = fx_decode(f64_bits(C.A[1][e]), base);
         }
     }
 }
@@ -607,9 +654,19 @@ cudaError_t launch_tile_recs(const ChareDev *ch, const TileDev *tiles, int64_t n
     return cudaGetLastError();
 }
 
-cudaError_t launch_face_copy(const ChareDev *ch, int nch, int parity, int face, int dir, double *buf, int64_t nx,
-                             int64_t ny, int64_t nz, const FmtDev *fmt, cudaStream_t s) {
-    k_face_copy<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, parity, face, dir, buf, nx, ny, nz, fmt);
+cudaError_t launch_face_copy(const ChareDev *ch, int px, int py, int pz, int parity, int face, int dir, double *buf,
+                             int64_t nx, int64_t ny, int64_t nz, uint64_t *vmax, FmtDev *fmt, uint32_t *wider,
+                             cudaStream_t s) {
+    const int axis = face / 2, p[3] = {px, py, pz}, step[3] = {1, px, px * py};
+    const int a = axis == 0 ? 1 : 0, b = axis == 2 ? 1 : 2;  // the face's own axes
+    const FaceChares on = {face % 2 ? (p[axis] - 1) * step[axis] : 0, step[a], p[a], step[b], p[b]};
+    const int64_t cells = axis == 0 ? ny * nz : axis == 1 ? nx * nz : nx * ny, n = (int64_t)on.na * on.nb;
+    // four cells a thread or more, up to two blocks for each SM (few, because
+    // an import's blocks are counted)
+    const int gy = (int)std::min<int64_t>(n, 304);
+    const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(304 / gy, (cells / n + 1023) / 1024));
+    k_face_copy<<<dim3(gx, gy), 256, 0, s>>>(ch, px * py * pz, on, parity, face, dir, buf, nx, ny, nz,
+                                             (unsigned long long *)vmax, fmt, wider);
     return cudaGetLastError();
 }
 
@@ -652,11 +709,10 @@ cudaError_t launch_scatter(const ChareDev *ch, int nch, int parity, int64_t nx, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_plain(const ChareDev *ch, int nch, FmtDev *fmt, cudaStream_t s) {
-    k_plain<<<dim3(io_grid_x(nch), io_grid_y(nch)), 256, 0, s>>>(ch, nch, fmt);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return cudaMemsetAsync(fmt, 0, sizeof *fmt, s);
+cudaError_t launch_refit(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, const uint64_t *vmax,
+                         FmtDev *fmt, cudaStream_t s) {
+    k_refit<<<608, 256, 0, s>>>(ch, nch, parity, nx, ny, nullptr, (const unsigned long long *)vmax, fmt);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ghost_refresh(const ChareDev *ch, int nch, int parity, cudaStream_t s) {

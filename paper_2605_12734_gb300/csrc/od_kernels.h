@@ -61,10 +61,14 @@ cudaError_t launch_tile_recs(const ChareDev *ch, const TileDev *tiles, int64_t n
 cudaError_t launch_init(const ChareDev *ch, int nch, int64_t gnx, int64_t gny, int64_t gnz, int64_t gx0,
                         int64_t gy0, int64_t gz0, uint64_t seed, int mode, int stencil, uint32_t base,
                         cudaStream_t s);
-// Domain-face exchange of a shard (od_face_copy): dir 0 copies the boundary
-// layer of parity p on face f into buf, dir 1 buf into the ghost layer.
-cudaError_t launch_face_copy(const ChareDev *ch, int nch, int parity, int face, int dir, double *buf, int64_t nx,
-                             int64_t ny, int64_t nz, const FmtDev *fmt, cudaStream_t s);
+// Domain-face exchange of a shard (od_face_copy) of px x py x pz chares: dir 0
+// copies the boundary layer of parity p on face f into buf, dir 1 buf into the
+// ghost layer.  vmax (null: the context never holds fixed-point words): an
+// import raises it to the face's largest value; *wider (mapped host memory) is
+// set to 1 when the field should take another format (launch_refit).
+cudaError_t launch_face_copy(const ChareDev *ch, int px, int py, int pz, int parity, int face, int dir, double *buf,
+                             int64_t nx, int64_t ny, int64_t nz, uint64_t *vmax, FmtDev *fmt, uint32_t *wider,
+                             cudaStream_t s);
 cudaError_t launch_pack(const ChareDev *ch, int c, int parity, int elems, cudaStream_t s);
 cudaError_t launch_unpack(const ChareDev *ch, int c, int parity, int slot, int elems, cudaStream_t s);
 // out[i] = *addr[i] for n device addresses (od_read_cells).
@@ -81,8 +85,9 @@ cudaError_t launch_arith(int op, const double *a, const double *b, double *out, 
 // format if that value asks for it.
 cudaError_t launch_scatter(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, int64_t nz,
                            const double *g, uint64_t *vmax, FmtDev *fmt, bool words, cudaStream_t s);
-// The whole context to plain doubles, for good.
-cudaError_t launch_plain(const ChareDev *ch, int nch, FmtDev *fmt, cudaStream_t s);
+// The field takes the format that *vmax asks for, if it has another.
+cudaError_t launch_refit(const ChareDev *ch, int nch, int parity, int64_t nx, int64_t ny, const uint64_t *vmax,
+                         FmtDev *fmt, cudaStream_t s);
 // Internal ghost layers of parity `parity` from the neighbours' boundaries.
 cudaError_t launch_ghost_refresh(const ChareDev *ch, int nch, int parity, cudaStream_t s);
 

@@ -177,3 +177,44 @@ def test_deep_rings_of_narrow_rows(od, path, stages):
     with od.Jacobi3D(1, 2048, 512, split=(1, 1, 1), seed=2, path=path, stages=stages) as s:
         s.step(3)
         assert same(s.read(), want)
+
+
+# faces fed before every step, whose values outgrow the window that the field's
+# words have, lie far below it, or ask for plain doubles: the whole field
+# follows, its other faces' shell included
+@pytest.mark.parametrize("path", PATHS)
+@pytest.mark.parametrize("scales", [(1.0, 0.5, 1.0), (1.0, 3e4, 1.0, 1e200, 1e-3), (1e-9, 2.0, 1e290, 1.0)])
+def test_faces_that_change_the_format(od, path, scales):
+    nx, ny, nz, seed = 36, 22, 29, 4
+    rng = np.random.default_rng(8)
+    P = oracle.init_padded(nx, ny, nz, seed, 1)
+    shell = [P[1:-1, 1:-1, 0], P[1:-1, 1:-1, -1], P[1:-1, 0, 1:-1], P[1:-1, -1, 1:-1], P[0, 1:-1, 1:-1],
+             P[-1, 1:-1, 1:-1]]
+    ghosts = [[a.copy() for a in shell], [a.copy() for a in shell]]  # of even and of odd steps' fields
+    with od.Jacobi3D(nx, ny, nz, split=(2, 2, 2), seed=seed, path=path) as s:
+        for t, scale in enumerate(scales * 2):
+            f = (5 * t) % 6
+            face = rng.random(shell[f].shape) * scale
+            if t % 3 == 2:
+                face[::4] *= -1.0
+            s.face_copy(f, 1, np.ascontiguousarray(face).ravel())
+            ghosts[t % 2][f][...] = face  # the field of this step's parity keeps it
+            for a, g in zip(shell, ghosts[t % 2]):
+                a[...] = g
+            s.step(1)
+            P[1:-1, 1:-1, 1:-1] = oracle.sweep(P.copy(), 1)[1:-1, 1:-1, 1:-1]
+            assert same(s.read(), oracle.interior(P)), (t, scale)
+
+
+def test_2d_faces_that_change_the_format(od):
+    nx, ny, seed = 120, 75, 4
+    rng = np.random.default_rng(8)
+    P = oracle.init_padded_2d(nx, ny, seed, 1)
+    with od.Jacobi2D(nx, ny, split=(2, 3), seed=seed, path="persistent") as s:
+        for scale in (1.0, 5e3, 1e240, 1.0):
+            face = rng.random(ny) * scale
+            s.face_copy(1, 1, face)
+            s.step(1)
+            P[1:-1, -1] = face
+            P = oracle.sweep_2d(P, 1)
+            assert same(s.read(), P[1:-1, 1:-1].ravel()), scale
