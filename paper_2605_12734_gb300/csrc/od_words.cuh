@@ -163,6 +163,12 @@ __device__ __forceinline__ uint32_t count_acq_rel(uint32_t *p) {
 constexpr int kRedoWarps = 16;  // of a CTA of up to 512 compute threads
 static_assert(kRedoWarps * 32 * 4 <= words_static_smem(256) - words_static_smem(128), "the planner's figure for it");
 
+// This warp's list: one array for every N that a kernel calls words_redo with.
+__device__ __forceinline__ int32_t *redo_list() {
+    __shared__ int32_t lists[kRedoWarps][32];
+    return lists[threadIdx.x >> 5];
+}
+
 template <int N>
 struct Offsets {
     int r[N];
@@ -172,8 +178,7 @@ template <int ST, int N>
 static __device__ __noinline__ void words_redo(const double *sd, const double *sc, const double *su, double *dpl,
                                                Offsets<N> rf, int pitch, uint32_t e0, bool rare) {
     constexpr bool k3D = ST == OD_STENCIL_3D7;
-    __shared__ int32_t lists[kRedoWarps][32];
-    int32_t *list = lists[threadIdx.x >> 5];
+    int32_t *list = redo_list();
     const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
     uint32_t number[N], total = 0;
 #pragma unroll

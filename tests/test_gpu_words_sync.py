@@ -85,3 +85,15 @@ def test_wait_limits_of_any_size(od, limit):
     with od.Jacobi3D(64, 64, 64, split=(2, 2, 2), seed=7, path="persistent", spin_limit_ns=limit) as s:
         s.step(40)
         assert same(s.read(), want)
+
+
+# rows of 500 cells in 256 x 2: the default ring fills the shared memory of
+# three CTAs an SM to within a kilobyte
+def test_resident_ctas_of_two_cells_a_thread(od):
+    torch = pytest.importorskip("torch")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    with od.Jacobi3D(500, 64, 64, split=(1, 1, 1), seed=2, path="persistent", threads=256, cells_per_thread=2,
+                     tile_z=4) as s:
+        s.step(3)
+        assert same(s.read(), oracle.solve(500, 64, 64, 2, 1, 3))
+        assert s.stats()["persistent_grid"] == 3 * sms
