@@ -60,13 +60,17 @@ __global__ void k_noalloc_step(const double *__restrict__ src, double *__restric
 
 // The same over fixed-point words (od_arith.cuh), for calls of several steps:
 // the field is turned into words once (two passes over it) and the last step
-// writes doubles.  A thread owns two cells of the plane, 256 apart in row-major
-// order, and sweeps them through a chunk of planes, so neighbouring planes are
-// found in L1; consecutive threads take consecutive cells whatever the row
-// length, so no lane is lost to ragged rows.  Bound by the integer ALU and L1:
-// 198^3, 20 steps: 1.52 ms with k_noalloc_step, 0.84 with this, whole calls (35 us
-// a step, 219 G updates/s).  Four cells a thread measured 0.94, one 0.98.
+// writes doubles.  The planes are cut into chunks, and the cells of a plane are
+// dealt over threads in order, two 256 apart to each, which it sweeps through a
+// chunk, so neighbouring planes are found in L1; consecutive threads take
+// consecutive cells whatever the row length, and planes that would not fill
+// their blocks' lanes share them, so few are lost.  Bound by the integer ALU
+// and L1: 198^3, 20 steps: 1.52 ms with k_noalloc_step, 0.84 with this, whole
+// calls (35 us a step, 219 G updates/s).  Four cells a thread measured 0.94, one
+// 0.98.  Planes of 3 cells (3 x 1 x 400000, 20 steps) 2.27 ms with
+// k_noalloc_step, 0.40 with this; with a chunk to each block 14.2.
 constexpr int kCells = 2, kBlock = 256;
+constexpr uint32_t kSms = 152;  // of a GB300
 
 __device__ unsigned long long g_vmax;  // bit pattern of the input's largest positive finite value
 
@@ -85,34 +89,59 @@ __global__ void k_noalloc_max(const double *__restrict__ u, uint32_t n) {
     if ((threadIdx.x & 31) == 0 && m) atomicMax(&g_vmax, m);
 }
 
-// Words of the whole input into `all` and of its Dirichlet shell into `shell`.
-__global__ void k_noalloc_encode(const double *__restrict__ u, double *__restrict__ all, double *__restrict__ shell,
-                                 uint32_t nx, uint32_t ny, uint32_t nz) {
-    const uint32_t base = od::fx_anchor(g_vmax), sx = nx + 2u, rows = (ny + 2u) * (nz + 2u);
-    for (uint32_t r = blockIdx.x; r < rows; r += gridDim.x) {
-        const uint32_t j = r % (ny + 2u), k = r / (ny + 2u);
-        const bool edge = j == 0u || j == ny + 1u || k == 0u || k == nz + 1u;
-        for (uint32_t i = threadIdx.x; i < sx; i += blockDim.x) {
-            const uint32_t c = r * sx + i;
-            const double w = od::f64_from(od::fx_encode(u[c], base));
-            all[c] = w;
-            if (edge || i == 0u || i == sx - 1u) shell[c] = w;
+// Every cell of the padded field: f(index, whether it is of the shell).  A row to
+// a block at a time, or, where rows are short or few, the cells in order (FLAT).
+template <bool FLAT, typename F>
+__device__ __forceinline__ void each_cell(uint32_t sx, uint32_t sy, uint32_t sz, F f) {
+    const uint32_t rows = sy * sz;
+    auto edge = [&](uint32_t r) {
+        const uint32_t j = r % sy, k = r / sy;
+        return j == 0u || j == sy - 1u || k == 0u || k == sz - 1u;
+    };
+    if (FLAT) {
+        for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < rows * sx; c += gridDim.x * blockDim.x) {
+            const uint32_t r = c / sx, i = c - r * sx;
+            f(c, i == 0u || i == sx - 1u || edge(r));
         }
+        return;
+    }
+    for (uint32_t r = blockIdx.x; r < rows; r += gridDim.x) {
+        const bool e = edge(r);
+        for (uint32_t i = threadIdx.x; i < sx; i += blockDim.x) f(r * sx + i, e || i == 0u || i == sx - 1u);
     }
 }
 
+// Words of the whole input into `all` and of its Dirichlet shell into `shell`.
+template <bool FLAT>
+__global__ void k_noalloc_encode(const double *__restrict__ u, double *__restrict__ all, double *__restrict__ shell,
+                                 uint32_t nx, uint32_t ny, uint32_t nz) {
+    const uint32_t base = od::fx_anchor(g_vmax);
+    each_cell<FLAT>(nx + 2u, ny + 2u, nz + 2u, [&](uint32_t c, bool edge) {
+        const double w = od::f64_from(od::fx_encode(u[c], base));
+        all[c] = w;
+        if (edge) shell[c] = w;
+    });
+}
+
+// OWN: a block has one chunk of planes (block y) of `planes`, the last one fewer.
+// Otherwise the cells of a plane times the chunks are dealt over the blocks in
+// order, and the last chunk begins early enough for `planes` of them (planes that
+// two chunks sweep get the same values from both).
+template <bool OWN>
 __global__ void __launch_bounds__(kBlock, 4)
     k_noalloc_words(const double *__restrict__ src, double *__restrict__ dst, uint32_t nx, uint32_t cells, uint32_t sx,
-                    uint32_t sxy, uint32_t nz, uint32_t chunk) {
+                    uint32_t sxy, uint32_t nz, uint32_t planes, uint32_t slots) {
     const uint32_t base = od::fx_anchor(g_vmax);
     int rf[kCells];
 #pragma unroll
     for (int m = 0; m < kCells; ++m) {
-        const uint32_t q0 = blockIdx.x * (kCells * kBlock) + m * kBlock + threadIdx.x;
-        const uint32_t q = q0 < cells ? q0 : 0u;  // past the end: cell 0 again, the same value to the same place
+        const uint32_t s0 = blockIdx.x * (kCells * kBlock) + m * kBlock + threadIdx.x;
+        const uint32_t s = s0 < slots ? s0 : 0u;  // past the end: slot 0 again, the same value to the same place
+        const uint32_t c = OWN ? 0u : s / cells, q = OWN ? s : s - c * cells;
         rf[m] = (int)((q / nx + 1u) * sx + q % nx + 1u);
+        if (!OWN) rf[m] += (int)(min(c * planes, nz - planes) * sxy);
     }
-    const uint32_t k0 = blockIdx.y * chunk, k1 = min(k0 + chunk, nz);
+    const uint32_t k0 = OWN ? blockIdx.y * planes : 0u, k1 = OWN ? min(k0 + planes, nz) : planes;
     for (uint32_t k = k0; k < k1; ++k) {
         const double *p = src + (size_t)k * sxy;
         od::tile::words_plane<kCells, OD_STENCIL_3D7, false>(p, p + sxy, p + 2u * sxy, dst + (size_t)(k + 1u) * sxy, rf,
@@ -121,17 +150,13 @@ __global__ void __launch_bounds__(kBlock, 4)
 }
 
 // The result's words to doubles, its shell from the input.
+template <bool FLAT>
 __global__ void k_noalloc_decode(const double *__restrict__ u, double *__restrict__ out, uint32_t nx, uint32_t ny,
                                  uint32_t nz) {
-    const uint32_t base = od::fx_anchor(g_vmax), sx = nx + 2u, rows = (ny + 2u) * (nz + 2u);
-    for (uint32_t r = blockIdx.x; r < rows; r += gridDim.x) {
-        const uint32_t j = r % (ny + 2u), k = r / (ny + 2u);
-        const bool edge = j == 0u || j == ny + 1u || k == 0u || k == nz + 1u;
-        for (uint32_t i = threadIdx.x; i < sx; i += blockDim.x) {
-            const uint32_t c = r * sx + i;
-            out[c] = edge || i == 0u || i == sx - 1u ? u[c] : od::fx_decode(od::f64_bits(out[c]), base);
-        }
-    }
+    const uint32_t base = od::fx_anchor(g_vmax);
+    each_cell<FLAT>(nx + 2u, ny + 2u, nz + 2u, [&](uint32_t c, bool edge) {
+        out[c] = edge ? u[c] : od::fx_decode(od::f64_bits(out[c]), base);
+    });
 }
 
 // Device address of the static scratch array on the current device, looked
@@ -162,23 +187,38 @@ od_status noalloc_words(const double *u_in, double *u_out, double *scratch, int6
     // the input's words start in the buffer that step 0 reads
     double *first = (iters - 1) % 2 == 0 ? u_out : scratch, *start = first == u_out ? scratch : u_out;
     const uint32_t rows = ((uint32_t)ny + 2u) * ((uint32_t)nz + 2u);
-    const uint32_t row_block = sx >= 256u ? 256u : sx > 64u ? 128u : 64u, row_grid = std::min<uint32_t>(rows, 65535u);
+    // (100000 x 3 x 5, 35 rows: 20 steps 0.57 ms by rows, 0.30 in order; 1 x 5003 x
+    // 211, rows of 3 cells: 0.62, 0.30)
+    const bool flat = sx < 64u || rows < 8u * kSms;
+    const uint32_t io_block = flat || sx >= 256u ? 256u : 128u;
+    const uint32_t io_grid = flat ? std::min<uint32_t>((n + 255u) / 256u, 64u * kSms) : std::min<uint32_t>(rows, 65535u);
     k_noalloc_reset<<<1, 1, 0, st>>>();
-    k_noalloc_max<<<std::min<uint32_t>((n + 1023u) / 1024u, 1216u), 256, 0, st>>>(u_in, n);
-    k_noalloc_encode<<<row_grid, row_block, 0, st>>>(u_in, start, first, (uint32_t)nx, (uint32_t)ny, (uint32_t)nz);
-    // chunks of planes: about four blocks for every one resident (4 per SM,
-    // 152 SMs); half, twice and four times as many measured slower
-    const uint32_t bx = (cells + kCells * kBlock - 1u) / (kCells * kBlock);
-        const uint32_t want = std::max<uint32_t>(1u, 2432u / bx);
-    const uint32_t chunk = ((uint32_t)nz + want - 1u) / want;
-    const dim3 grid(bx, ((uint32_t)nz + chunk - 1u) / chunk);
+    k_noalloc_max<<<std::min<uint32_t>((n + 1023u) / 1024u, 8u * kSms), 256, 0, st>>>(u_in, n);
+    auto encode = flat ? k_noalloc_encode<true> : k_noalloc_encode<false>;
+    auto decode = flat ? k_noalloc_decode<true> : k_noalloc_decode<false>;
+    encode<<<io_grid, io_block, 0, st>>>(u_in, start, first, (uint32_t)nx, (uint32_t)ny, (uint32_t)nz);
+    // chunks of planes: about four blocks for every one resident (4 per SM); half,
+    // twice and four times as many measured slower.  A block has a chunk of its
+    // own unless that leaves a sixteenth of the lanes idle (dealt in order, planes
+    // of 4000 to 40000 cells ran up to 7 % slower).
+    auto blocks = [](uint32_t m) { return (m + kCells * kBlock - 1u) / (kCells * kBlock); };
+    const bool own = blocks(cells) * (kCells * kBlock) <= cells + cells / 16u;
+    const uint32_t want = std::max<uint32_t>(1u, own ? 16u * kSms / blocks(cells) : 16u * kSms * kCells * kBlock / cells);
+    const uint32_t planes = ((uint32_t)nz + want - 1u) / want, chunks = ((uint32_t)nz + planes - 1u) / planes;
+    const uint32_t slots = own ? cells : cells * chunks;
+    const dim3 grid(blocks(slots), own ? chunks : 1u);
     const double *src = start;
     for (int32_t t = 0; t < iters; ++t) {
         double *dst = ((iters - 1 - t) % 2 == 0) ? u_out : scratch;
-        k_noalloc_words<<<grid, kBlock, 0, st>>>(src, dst, (uint32_t)nx, cells, sx, sxy, (uint32_t)nz, chunk);
+        if (own)
+            k_noalloc_words<true>
+                <<<grid, kBlock, 0, st>>>(src, dst, (uint32_t)nx, cells, sx, sxy, (uint32_t)nz, planes, slots);
+        else
+            k_noalloc_words<false>
+                <<<grid, kBlock, 0, st>>>(src, dst, (uint32_t)nx, cells, sx, sxy, (uint32_t)nz, planes, slots);
         src = dst;
     }
-    k_noalloc_decode<<<row_grid, row_block, 0, st>>>(u_in, u_out, (uint32_t)nx, (uint32_t)ny, (uint32_t)nz);
+    decode<<<io_grid, io_block, 0, st>>>(u_in, u_out, (uint32_t)nx, (uint32_t)ny, (uint32_t)nz);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(OD_ECUDA, std::string("od_jacobi_noalloc: ") + cudaGetErrorString(e));
     return OD_OK;
@@ -207,10 +247,12 @@ extern "C" OD_API od_status od_jacobi_noalloc(const double *u_in, double *u_out,
     // Calls of several steps on a field that fills the GPU sweep words.  A step
     // takes 4.6 ps a cell then instead of 9.4, the conversions 6 ps a cell and
     // four launches; below a million cells a step is latency either way.
-    // Measured, us: 198^3 x 2 208 with words, 211 without, x 3 243 / 284, x 20
-    // 844 / 1520; 500 x 100 x 100 x 3 162 / 177; 64^3 x 20 151 / 144.
+    // Measured, us: 198^3 x 2 208 with words, 211 without, x 3 238 / 283, x 20
+    // 838 / 1506; 500 x 100 x 100 x 3 162 / 177; 64^3 x 20 151 / 144.  One plane
+    // or two are mostly shell and find no plane again: 1100 x 1000 x 1 x 20 296 /
+    // 280, 1400 x 1400 x 2 x 3 181 / 169, x 6 260 / 274.
     const int64_t cells = nx * ny * nz;
-    if (iters >= 3 && cells >= (1 << 20) && cells * (iters - 1) >= 6000000)
+    if (iters >= (nz == 2 ? 6 : 3) && nz > 1 && cells >= (1 << 20) && cells * (iters - 1) >= 6000000)
         return noalloc_words(u_in, u_out, scratch, nx, ny, nz, iters, st);
     // Both buffers start as the input, so both hold the Dirichlet shell and
     // nothing of an earlier call survives in the scratch.

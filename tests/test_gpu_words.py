@@ -218,3 +218,22 @@ def test_2d_faces_that_change_the_format(od):
             P[1:-1, -1] = face
             P = oracle.sweep_2d(P, 1)
             assert same(s.read(), P[1:-1, 1:-1].ravel()), scale
+
+
+# planes of few cells share blocks, the last chunk of planes overlaps the one
+# before; short rows and few rows are converted cell by cell; one and two planes
+@pytest.mark.parametrize("dims", [(8, 8, 20011), (2, 1500, 400), (60000, 3, 7), (1, 1, 930000), (24, 22, 2503),
+                                  (1100, 600, 2), (1200, 1001, 1)])
+@pytest.mark.parametrize("kind", ["uniform", "tiny"])
+def test_allocation_free_entry_of_narrow_and_flat_fields(od, dims, kind):
+    import torch
+    nx, ny, nz = dims
+    rng = np.random.default_rng(nx)
+    P = field(kind, (nx + 2) * (ny + 2) * (nz + 2), rng).reshape(nz + 2, ny + 2, nx + 2)
+    for iters in (7, 10):
+        want = oracle.sweep(P.copy(), iters)
+        want[:, :, [0, -1]], want[:, [0, -1]], want[[0, -1]] = P[:, :, [0, -1]], P[:, [0, -1]], P[[0, -1]]
+        u = torch.from_numpy(P.ravel().copy()).to("cuda:0")
+        out = torch.full_like(u, -1.0)
+        od.jacobi_noalloc(u, out, nx, ny, nz, iters)
+        assert same(out.cpu().numpy().reshape(P.shape), want), iters
