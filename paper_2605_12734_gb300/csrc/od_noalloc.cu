@@ -35,7 +35,11 @@ static __device__ __align__(256) double g_scratch[kScratchDoubles];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
-double *g_scratch_ptr[kMaxDevices] = {nullptr};
+struct Statics {  // device addresses of the static arrays of a device
+    double *scratch;
+    uint32_t *chosen, *base;
+};
+Statics g_statics[kMaxDevices] = {};
 od_status set_error(od_status s, const std::string &m) { return od::set_last_error(s, m); }
 
 // One step over the interior of a padded field (x fastest, row length nx+2):
@@ -72,11 +76,45 @@ __global__ void k_noalloc_step(const double *__restrict__ src, double *__restric
 constexpr int kCells = 2, kBlock = 256;
 constexpr uint32_t kSms = 152;  // of a GB300
 
-__device__ unsigned long long g_vmax;  // bit pattern of the input's largest positive finite value
+// Of a call, beside the static scratch: the bit pattern of the input's largest
+// positive finite value and the blocks that have looked for it, both left at
+// zero for the next call, and the format the sweep runs in, a base exponent or 0
+// for doubles: chosen into g_base, copied to c_base, from which the sweep reads it
+// through the constant cache (a load from g_base at the head of every block cost
+// 198^3 a microsecond a step).
+__device__ unsigned long long g_vmax;
+__device__ uint32_t g_done, g_base;
+__constant__ uint32_t c_base;
 
-__global__ void k_noalloc_reset() { g_vmax = 0; }
+// 256 updates spread over the field (a Weyl sequence of the golden ratio): the
+// lowest exponent of the six operands and the result in the low half (0xFFFF: all
+// zero), whether one of them is no positive finite value, and whether the update
+// stays in a window of its own.
+constexpr uint32_t kNoWord = 1u << 31, kOwnWindow = 1u << 30;
+__device__ uint32_t g_sample[256];
 
-__global__ void k_noalloc_max(const double *__restrict__ u, uint32_t n) {
+__device__ uint32_t sample_update(const double *u, uint32_t t, uint32_t nx, uint32_t ny, uint32_t nz) {
+    const uint32_t sx = nx + 2u, sxy = sx * (ny + 2u), cells = nx * ny * nz;
+    const uint32_t q = (uint32_t)(((uint64_t)((t + 1u) * 0x9E3779B9u) * cells) >> 32), r = q / nx;
+    const double *c = u + (size_t)(r / ny + 1u) * sxy + (r % ny + 1u) * sx + (q - r * nx) + 1u;
+    double x[7] = {c[-1], c[1], *(c - sx), c[sx], *(c - sxy), c[sxy], 0.0};
+    bool own;
+    od::jacobi_update_fast<2>(x[0], x[1], x[2], x[3], x[4], x[5], own);
+    x[6] = od::jacobi_update_ieee<true>(x[0], x[1], x[2], x[3], x[4], x[5]);
+    uint32_t low = 0xFFFFu, flags = own ? kOwnWindow : 0u;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        const uint64_t b = od::f64_bits(x[i]);
+        const uint32_t e = (uint32_t)(b >> 52);
+        if (b != 0u) low = min(low, e);
+        if (e >= 0x7FFu) flags |= kNoWord;
+    }
+    return low | flags;
+}
+
+__global__ void __launch_bounds__(256) k_noalloc_max(const double *__restrict__ u, uint32_t nx, uint32_t ny, uint32_t nz) {
+    const uint32_t n = (nx + 2u) * (ny + 2u) * (nz + 2u);
+    if (blockIdx.x == 0) g_sample[threadIdx.x] = sample_update(u, threadIdx.x, nx, ny, nz);
     unsigned long long m = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const unsigned long long b = od::f64_bits(u[i]);
@@ -87,6 +125,29 @@ __global__ void k_noalloc_max(const double *__restrict__ u, uint32_t n) {
         m = w > m ? w : m;
     }
     if ((threadIdx.x & 31) == 0 && m) atomicMax(&g_vmax, m);
+    // The last block to finish chooses the format.  Words have one window for the
+    // whole field and an update outside it costs about 2.6 times one inside;
+    // doubles take a window for each update, the six operands within 8 binades, at
+    // twice the cost, and 7.7 times where they are not (198^3, us a step: 36, 94,
+    // 73, 277).  So a smooth field over many binades, or one with a single large
+    // value, sweeps doubles, and a signed one words.  (20 steps of 198^3 from such a
+    // field: 1.74 ms over words, 1.45 this way, 1.49 by k_noalloc_step.)
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&g_done, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const uint32_t base = od::fx_anchor(*(volatile unsigned long long *)&g_vmax);
+    const uint32_t sample = *(volatile uint32_t *)&g_sample[threadIdx.x];
+    const int words = __syncthreads_count((sample & kNoWord) == 0u && (sample & 0xFFFFu) >= base);
+    const int own = __syncthreads_count((sample & kOwnWindow) != 0u);
+    if (threadIdx.x == 0) {
+        g_base = 73 * own + 277 * (256 - own) < 36 * words + 94 * (256 - words) ? 0u : base;
+        g_vmax = 0ull;
+        g_done = 0u;
+    }
 }
 
 // Every cell of the padded field: f(index, whether it is of the shell).  A row to
@@ -115,7 +176,7 @@ __device__ __forceinline__ void each_cell(uint32_t sx, uint32_t sy, uint32_t sz,
 template <bool FLAT>
 __global__ void k_noalloc_encode(const double *__restrict__ u, double *__restrict__ all, double *__restrict__ shell,
                                  uint32_t nx, uint32_t ny, uint32_t nz) {
-    const uint32_t base = od::fx_anchor(g_vmax);
+    const uint32_t base = c_base;
     each_cell<FLAT>(nx + 2u, ny + 2u, nz + 2u, [&](uint32_t c, bool edge) {
         const double w = od::f64_from(od::fx_encode(u[c], base));
         all[c] = w;
@@ -131,7 +192,7 @@ template <bool OWN>
 __global__ void __launch_bounds__(kBlock, 4)
     k_noalloc_words(const double *__restrict__ src, double *__restrict__ dst, uint32_t nx, uint32_t cells, uint32_t sx,
                     uint32_t sxy, uint32_t nz, uint32_t planes, uint32_t slots) {
-    const uint32_t base = od::fx_anchor(g_vmax);
+    const uint32_t base = c_base;
     int rf[kCells];
 #pragma unroll
     for (int m = 0; m < kCells; ++m) {
@@ -142,6 +203,18 @@ __global__ void __launch_bounds__(kBlock, 4)
         if (!OWN) rf[m] += (int)(min(c * planes, nz - planes) * sxy);
     }
     const uint32_t k0 = OWN ? blockIdx.y * planes : 0u, k1 = OWN ? min(k0 + planes, nz) : planes;
+    if (base == 0u) {  // doubles, as k_noalloc_step
+#pragma unroll 1
+        for (uint32_t k = k0; k < k1; ++k)
+#pragma unroll
+            for (int m = 0; m < kCells; ++m) {
+                const double *c = src + (size_t)(k + 1u) * sxy + rf[m];
+                dst[(size_t)(k + 1u) * sxy + rf[m]] =
+                    od::jacobi_update<2>(c[-1], c[1], *(c - sx), c[sx], *(c - sxy), c[sxy]);
+            }
+        return;
+    }
+#pragma unroll 1
     for (uint32_t k = k0; k < k1; ++k) {
         const double *p = src + (size_t)k * sxy;
         od::tile::words_plane<kCells, OD_STENCIL_3D7, false>(p, p + sxy, p + 2u * sxy, dst + (size_t)(k + 1u) * sxy, rf,
@@ -153,38 +226,45 @@ __global__ void __launch_bounds__(kBlock, 4)
 template <bool FLAT>
 __global__ void k_noalloc_decode(const double *__restrict__ u, double *__restrict__ out, uint32_t nx, uint32_t ny,
                                  uint32_t nz) {
-    const uint32_t base = od::fx_anchor(g_vmax);
+    const uint32_t base = c_base;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // (again: calls that overlapped, against the rules, may have left them)
+        g_vmax = 0ull;
+        g_done = 0u;
+    }
+    if (base == 0u) return;  // doubles, and the shell is there from the start
     each_cell<FLAT>(nx + 2u, ny + 2u, nz + 2u, [&](uint32_t c, bool edge) {
         out[c] = edge ? u[c] : od::fx_decode(od::f64_bits(out[c]), base);
     });
 }
 
-// Device address of the static scratch array on the current device, looked
-// up once per device (the symbol's name is only a host-side stand-in).
-od_status scratch_for_current_device(double **out) {
+// Device addresses of the static arrays on the current device, looked up once
+// per device (a symbol's name is only a host-side stand-in).
+od_status statics_for_current_device(Statics *out) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return set_error(OD_ECUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(e));
     if (dev < 0 || dev >= kMaxDevices) return set_error(OD_EINVAL, "device ordinal out of range");
     std::lock_guard<std::mutex> lock(g_mu);
-    if (!g_scratch_ptr[dev]) {
-        void *p = nullptr;
-        e = cudaGetSymbolAddress(&p, g_scratch);
-        if (e != cudaSuccess || !p)
+    if (!g_statics[dev].scratch) {
+        void *p[3] = {nullptr, nullptr, nullptr};
+        e = cudaGetSymbolAddress(&p[0], g_scratch);
+        if (e == cudaSuccess) e = cudaGetSymbolAddress(&p[1], g_base);
+        if (e == cudaSuccess) e = cudaGetSymbolAddress(&p[2], c_base);
+        if (e != cudaSuccess || !p[0] || !p[1] || !p[2])
             return set_error(OD_ECUDA, std::string("cudaGetSymbolAddress(scratch): ") + cudaGetErrorString(e));
-        g_scratch_ptr[dev] = (double *)p;
+        g_statics[dev] = {(double *)p[0], (uint32_t *)p[1], (uint32_t *)p[2]};
     }
-    *out = g_scratch_ptr[dev];
+    *out = g_statics[dev];
     return OD_OK;
 }
 
-
-od_status noalloc_words(const double *u_in, double *u_out, double *scratch, int64_t nx, int64_t ny, int64_t nz,
+od_status noalloc_words(const double *u_in, double *u_out, const Statics &dev, int64_t nx, int64_t ny, int64_t nz,
                         int32_t iters, cudaStream_t st) {
     const uint32_t sx = (uint32_t)nx + 2u, sxy = sx * ((uint32_t)ny + 2u), n = sxy * ((uint32_t)nz + 2u);
     const uint32_t cells = (uint32_t)(nx * ny);
     // step t writes u_out when iters-1-t is even, so the last step lands there;
     // the input's words start in the buffer that step 0 reads
+    double *const scratch = dev.scratch;
     double *first = (iters - 1) % 2 == 0 ? u_out : scratch, *start = first == u_out ? scratch : u_out;
     const uint32_t rows = ((uint32_t)ny + 2u) * ((uint32_t)nz + 2u);
     // (100000 x 3 x 5, 35 rows: 20 steps 0.57 ms by rows, 0.30 in order; 1 x 5003 x
@@ -192,8 +272,10 @@ od_status noalloc_words(const double *u_in, double *u_out, double *scratch, int6
     const bool flat = sx < 64u || rows < 8u * kSms;
     const uint32_t io_block = flat || sx >= 256u ? 256u : 128u;
     const uint32_t io_grid = flat ? std::min<uint32_t>((n + 255u) / 256u, 64u * kSms) : std::min<uint32_t>(rows, 65535u);
-    k_noalloc_reset<<<1, 1, 0, st>>>();
-    k_noalloc_max<<<std::min<uint32_t>((n + 1023u) / 1024u, 8u * kSms), 256, 0, st>>>(u_in, n);
+    k_noalloc_max<<<std::min<uint32_t>((n + 1023u) / 1024u, 8u * kSms), 256, 0, st>>>(u_in, (uint32_t)nx, (uint32_t)ny,
+                                                                                      (uint32_t)nz);
+    cudaError_t e = cudaMemcpyAsync(dev.base, dev.chosen, sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess) return set_error(OD_ECUDA, std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
     auto encode = flat ? k_noalloc_encode<true> : k_noalloc_encode<false>;
     auto decode = flat ? k_noalloc_decode<true> : k_noalloc_decode<false>;
     encode<<<io_grid, io_block, 0, st>>>(u_in, start, first, (uint32_t)nx, (uint32_t)ny, (uint32_t)nz);
@@ -219,7 +301,7 @@ od_status noalloc_words(const double *u_in, double *u_out, double *scratch, int6
         src = dst;
     }
     decode<<<io_grid, io_block, 0, st>>>(u_in, u_out, (uint32_t)nx, (uint32_t)ny, (uint32_t)nz);
-    const cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(OD_ECUDA, std::string("od_jacobi_noalloc: ") + cudaGetErrorString(e));
     return OD_OK;
 }
@@ -240,9 +322,10 @@ extern "C" OD_API od_status od_jacobi_noalloc(const double *u_in, double *u_out,
     const uintptr_t a0 = (uintptr_t)u_in, b0 = (uintptr_t)u_out;
     if (a0 < b0 + bytes && b0 < a0 + bytes)
         return set_error(OD_EINVAL, "od_jacobi_noalloc: input and output fields overlap");
-    double *scratch = nullptr;
-    od_status s = scratch_for_current_device(&scratch);
+    Statics dev = {};
+    od_status s = statics_for_current_device(&dev);
     if (s != OD_OK) return s;
+    double *const scratch = dev.scratch;
     cudaStream_t st = (cudaStream_t)stream;
     // Calls of several steps on a field that fills the GPU sweep words.  A step
     // takes 4.6 ps a cell then instead of 9.4, the conversions 6 ps a cell and
@@ -253,7 +336,7 @@ extern "C" OD_API od_status od_jacobi_noalloc(const double *u_in, double *u_out,
     // 280, 1400 x 1400 x 2 x 3 181 / 169, x 6 260 / 274.
     const int64_t cells = nx * ny * nz;
     if (iters >= (nz == 2 ? 6 : 3) && nz > 1 && cells >= (1 << 20) && cells * (iters - 1) >= 6000000)
-        return noalloc_words(u_in, u_out, scratch, nx, ny, nz, iters, st);
+        return noalloc_words(u_in, u_out, dev, nx, ny, nz, iters, st);
     // Both buffers start as the input, so both hold the Dirichlet shell and
     // nothing of an earlier call survives in the scratch.
     cudaError_t e = cudaMemcpyAsync(u_out, u_in, bytes, cudaMemcpyDeviceToDevice, st);

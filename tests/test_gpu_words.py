@@ -237,3 +237,37 @@ def test_allocation_free_entry_of_narrow_and_flat_fields(od, dims, kind):
         out = torch.full_like(u, -1.0)
         od.jacobi_noalloc(u, out, nx, ny, nz, iters)
         assert same(out.cpu().numpy().reshape(P.shape), want), iters
+
+
+# fields whose updates each fit a window of their own but not the field's one: the
+# sweep keeps doubles, after a call that did not and before one that does not
+@pytest.mark.parametrize("dims", [(131, 127, 65), (12, 10, 10007)])
+@pytest.mark.parametrize("kind", ["smooth", "hot", "signed", "nan"])
+def test_allocation_free_entry_chooses_its_format(od, dims, kind):
+    import torch
+    nx, ny, nz = dims
+    shape = (nz + 2, ny + 2, nx + 2)
+    rng = np.random.default_rng(nx)
+
+    def call(P, iters):
+        want = oracle.sweep(P.copy(), iters)
+        want[:, :, [0, -1]], want[:, [0, -1]], want[[0, -1]] = P[:, :, [0, -1]], P[:, [0, -1]], P[[0, -1]]
+        u = torch.from_numpy(P.ravel().copy()).to("cuda:0")
+        out = torch.full_like(u, -1.0)
+        od.jacobi_noalloc(u, out, nx, ny, nz, iters)
+        return out.cpu().numpy().reshape(shape), want
+
+    plain = rng.random(shape)
+    P = rng.random(shape)
+    if kind == "smooth":
+        P = np.exp2(-90.0 * np.arange(nz + 2) / nz)[:, None, None] * (0.9 + 0.1 * P)
+    elif kind == "hot":
+        P[nz // 2, 0, :] = 1e9
+    elif kind == "signed":
+        P -= 0.5
+    else:
+        P[nz // 2, 5, 5] = np.nan
+    for field_, iters in ((plain, 8), (P, 8), (P, 9), (plain, 9)):
+        got, want = call(field_, iters)
+        assert np.array_equal(np.isnan(got), np.isnan(want))
+        assert same(np.nan_to_num(got), np.nan_to_num(want)), iters
