@@ -1219,8 +1219,12 @@ od_status od_face_copy(od_ctx *c, int32_t face, int32_t dir, double *buf, int32_
     const int64_t n = f < 2 ? p.ny * p.nz : f < 4 ? p.nx * p.nz : p.nx * p.ny;
     DeviceGuard dg(c->device);
     const int par = (int)(c->steps & 1);
-    if (dir == 1 && c->words && !c->wider) {  // the first import
-        OD_CUDA(cudaHostAlloc(&c->wider, sizeof *c->wider, cudaHostAllocMapped));
+    if (dir == 1 && c->words && !c->wider) {  // the first import, perhaps under a stream capture
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        OD_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+        const cudaError_t e = cudaHostAlloc(&c->wider, sizeof *c->wider, cudaHostAllocMapped);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        OD_CUDA(e);
         *c->wider = 0u;
     }
     // the copy between the device-visible buffer b and the field

@@ -271,3 +271,44 @@ def test_allocation_free_entry_chooses_its_format(od, dims, kind):
         got, want = call(field_, iters)
         assert np.array_equal(np.isnan(got), np.isnan(want))
         assert same(np.nan_to_num(got), np.nan_to_num(want)), iters
+
+
+# a context's first face import may be part of a stream capture
+def test_first_face_import_under_capture(od):
+    import torch
+    nx, ny, nz, seed = 24, 20, 16, 3
+    st = torch.cuda.Stream()
+    face = torch.from_numpy(np.random.default_rng(1).random(ny * nz) * 7.0).cuda()
+    P = oracle.init_padded(nx, ny, nz, seed, 1)
+    with od.Jacobi3D(nx, ny, nz, split=(2, 2, 1), seed=seed, path="persistent", stream=st.cuda_stream) as s:
+        s.sync()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            s.face_copy(0, 1, face)
+        g.replay()
+        torch.cuda.synchronize()
+        P[1:-1, 1:-1, 0] = face.cpu().numpy().reshape(nz, ny)
+        s.step(1)
+        assert same(s.read(), oracle.interior(oracle.sweep(P, 1)))
+
+
+# most of a signed field's cells leave the window; NaN spreads by one cell a step
+@pytest.mark.parametrize("path", PATHS)
+@pytest.mark.parametrize("threads,cpt", [(128, 2), (128, 4), (256, 4), (512, 2)])
+def test_signed_fields_and_nan(od, path, threads, cpt):
+    nx, ny, nz, seed, iters = 62, 31, 24, 5, 5
+    rng = np.random.default_rng(threads + cpt)
+    u = rng.random(nx * ny * nz) - 0.5
+    kw = dict(split=(2, 2, 2), seed=seed, path=path, threads=threads, cells_per_thread=cpt)
+    with od.Jacobi3D(nx, ny, nz, **kw) as s:
+        s.write(u)
+        s.step(iters)
+        assert same(s.read(), solve_from(nx, ny, nz, seed, u, iters))
+        u[nx * ny * 11 + 7] = np.nan
+        s.write(u)
+        s.step(2)
+        s.step(1)
+        got, want = s.read(), solve_from(nx, ny, nz, seed, u, 3)
+        assert np.array_equal(np.isnan(got), np.isnan(want)) and np.isnan(want).sum() > 20
+        assert same(np.nan_to_num(got), np.nan_to_num(want))
