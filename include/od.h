@@ -165,9 +165,11 @@ typedef struct od_config {
                                     other / every fourth cell, 12 on the rest.
                                     Mode 12 keeps the field itself as words of
                                     such a window where it can (from od_create
-                                    or od_write on; until the field or a face
-                                    fed to it reaches 2^757) and then needs no
-                                    FP64 add.
+                                    or od_write on) and then needs no FP64 add.
+                                    Once the field or a face fed to it has
+                                    reached 2^757 it holds plain doubles, whose
+                                    updates all run in the IEEE form: the same
+                                    bits at about half the speed.
                                     2D: 12 one FP64 add and two window adds,
                                     13 none and three, 14 the two mixed, 15
                                     two FP64 adds and one window add.  -1 =
@@ -207,7 +209,12 @@ typedef struct od_plan_info {
     int64_t face_cells_internal;   /* ghost cells fed by a neighbour, summed
                                       over chares (each shared face twice) */
     int64_t face_cells_dirichlet;  /* ghost cells on the domain shell */
-    uint64_t arena_bytes;          /* device bytes od_create needs */
+    uint64_t arena_bytes;          /* device bytes od_create needs: both parities of
+                                      every chare with its ghosts (a row takes 4
+                                      doubles more than its cells where these are a
+                                      multiple of 4, 2 or 3 otherwise), its face
+                                      buffers, and some 80 bytes a tile, 340 in the
+                                      default arithmetic (its tile records) */
     double bytes_per_step;         /* algorithmic HBM bytes per iteration:
                                       16*cells + 16*face_internal + 8*face_dirichlet */
     int32_t tile_y, tile_z;        /* largest tile used: rows, planes */
@@ -488,7 +495,8 @@ OD_API od_status od_bench_launch_rate(int32_t device, int32_t host_threads, int3
 typedef struct od_server od_server;
 
 typedef struct od_server_config {
-    uint64_t hbm_budget_bytes;   /* device memory for all resident jobs */
+    uint64_t hbm_budget_bytes;   /* device memory for all resident jobs; each
+                                    takes its od_plan_info.arena_bytes */
     int32_t max_active;          /* jobs resident at once (0 = no limit) */
     int32_t max_jobs_per_launch; /* batched mode: batch table size (0 = 256) */
     int32_t device;

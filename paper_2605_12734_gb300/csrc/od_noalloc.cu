@@ -74,7 +74,7 @@ __global__ void k_noalloc_step(const double *__restrict__ src, double *__restric
 // 0.98.  Planes of 3 cells (3 x 1 x 400000, 20 steps) 2.27 ms with
 // k_noalloc_step, 0.40 with this; with a chunk to each block 14.2.
 constexpr int kCells = 2, kBlock = 256;
-constexpr uint32_t kSms = 152;  // of a GB300
+constexpr uint32_t kSms = od::kSms;
 
 // Of a call, beside the static scratch: the bit pattern of the input's largest
 // positive finite value and the blocks that have looked for it, both left at

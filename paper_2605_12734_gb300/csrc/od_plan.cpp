@@ -196,7 +196,7 @@ static void words_shape(const Plan &p, bool fused, int32_t stages, int32_t *thre
         return;
     int64_t nt = 0, nd = 0;
     if (fused) count_tiles(p, 1024, 32, &nt, &nd);
-    if (!fused || nt >= 3 * 3 * 152) *threads = 256;  // three resident CTAs an SM
+    if (!fused || nt >= 3 * 3 * kSms) *threads = 256;  // three resident CTAs an SM
 }
 
 // Planes (2D: rows) per tile that a context's sweep over words runs with when
@@ -380,7 +380,7 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
                         rows += v * ((double)by / slabs);
                         tiles += (double)slabs * chunks;
                     }
-            const double resident = 0.5 * 152.0 * (1280 / shapes[i][0]);
+            const double resident = 0.5 * kSms * (1280 / shapes[i][0]);
             const double score = used / cells * (1.0 - 0.2 / (rows / used)) *
                                  (fill_gpu ? std::min(1.0, tiles / resident) : 1.0);
             if (i == 0) base = score;

@@ -15,6 +15,7 @@ namespace od {
 // Default arithmetic: the anchored integer window, with the field kept as
 // fixed-point words where the context allows it (od_arith.cuh).
 constexpr int32_t kDefaultArith = 12;
+constexpr int kSms = 152;        // SMs of a GB300, for which the planner's rules were measured
 constexpr int32_t kFxMode = 16;  // the tile kernels' mode for mode 12 over such words
 // Resident CTAs per SM of the kernels over words (od_words.cuh): their
 // register budget a thread, for NT compute threads and the producer warp.
