@@ -382,7 +382,7 @@ constexpr int kIoRows = 4;
 // to export, and g stays as it is.
 __global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, double *g, const FmtDev *fmt,
                          const ErrDev *err) {
-    if (err && err->code != 0) return;
+    const bool failed = err && err->code != 0;  // (looked at after the first cells are loaded)
     const uint32_t base = fmt->base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int c = blockIdx.y; c < nch; c += gridDim.y) {
@@ -403,6 +403,7 @@ __global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t
                 double v[kIoRows];
 #pragma unroll
                 for (int u = 0; u < kIoRows; ++u) v[u] = src[u][i];
+                if (failed) return;
 #pragma unroll
                 for (int u = 0; u < kIoRows; ++u)
                     dst[u][i] = fx_decode(f64_bits(v[u]), base);  // a repeated row stores the same value
