@@ -69,8 +69,8 @@ __global__ void k_noalloc_step(const double *__restrict__ src, double *__restric
 // chunk, so neighbouring planes are found in L1; consecutive threads take
 // consecutive cells whatever the row length, and planes that would not fill
 // their blocks' lanes share them, so few are lost.  Bound by the integer ALU
-// and L1: 198^3, 20 steps: 1.52 ms with k_noalloc_step, 0.84 with this, whole
-// calls (35 us a step, 219 G updates/s).  Four cells a thread measured 0.94, one
+// and L1: 198^3, 20 steps: 1.52 ms with k_noalloc_step, 0.86 with this, whole
+// calls (36 us a step, 216 G updates/s).  Four cells a thread measured 0.94, one
 // 0.98.  Planes of 3 cells (3 x 1 x 400000, 20 steps) 2.27 ms with
 // k_noalloc_step, 0.40 with this; with a chunk to each block 14.2.
 constexpr int kCells = 2, kBlock = 256;
@@ -330,8 +330,8 @@ extern "C" OD_API od_status od_jacobi_noalloc(const double *u_in, double *u_out,
     // Calls of several steps on a field that fills the GPU sweep words.  A step
     // takes 4.6 ps a cell then instead of 9.4, the conversions 6 ps a cell and
     // four launches; below a million cells a step is latency either way.
-    // Measured, us: 198^3 x 2 208 with words, 211 without, x 3 238 / 283, x 20
-    // 838 / 1506; 500 x 100 x 100 x 3 162 / 177; 64^3 x 20 151 / 144.  One plane
+    // Measured, us: 198^3 x 2 208 with words, 211 without, x 3 234 / 283, x 20
+    // 858 / 1506; 500 x 100 x 100 x 3 162 / 177; 64^3 x 20 151 / 144.  One plane
     // or two are mostly shell and find no plane again: 1100 x 1000 x 1 x 20 296 /
     // 280, 1400 x 1400 x 2 x 3 181 / 169, x 6 260 / 274.
     const int64_t cells = nx * ny * nz;

@@ -258,8 +258,8 @@ od_status build_plan(const od_config *cfg, Plan *P, std::string *err, bool fill_
     p.tile_y = cfg->tile_y;
     p.tile_z = cfg->tile_z;
     // default: the anchored window, the field kept as words of it (512^3 in
-    // 4096 chares: 303 G updates/s, against 205 with plain doubles and two FP64
-    // adds; 32768^2: 416 against 345 with one)
+    // 4096 chares: 305 G updates/s, against 205 with plain doubles and two FP64
+    // adds; 32768^2: 417 against 345 with one)
     p.amode = cfg->arith >= 0 ? cfg->arith : kDefaultArith;
     if (p.amode > 15) {
         *err = "arith must be in [0, 15] (or -1 for the default)";

@@ -28,7 +28,8 @@
 // producer that alternates strictly between issuing and finishing planes,
 // 0.541 event-driven, 0.524 with one 256-byte record per tile instead of five
 // dependent table reads, 0.489 with 6 ring slots (0.456 with the roundings left
-// out), 0.460 with rows of whole sectors (od_plan.cpp), 0.443 with 256 x 4.  Two-dimensional,
+// out), 0.460 with rows of whole sectors (od_plan.cpp), 0.443 with 256 x 4, 0.441 with
+// conversions that select (od_arith.cuh).  Two-dimensional,
 // 16384^2: 0.76 to 0.65.  What bounds it: at 32^3 chares the traffic (2.39 GB a
 // step, 0.79 of the copy bandwidth) and the ALU pipe (62 % busy, issue 67 %)
 // together; in two dimensions the copy bandwidth (0.99 of it).  A fused step on
