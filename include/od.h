@@ -304,7 +304,8 @@ OD_API od_status od_sync(od_ctx *ctx);
  * context's device; otherwise host memory: pinned (page-locked) host memory
  * is written in place by the gather kernel over the host link, pageable
  * memory through a device staging buffer of nx*ny*nz doubles allocated on
- * the first such read or write and kept.  Synchronises the stream. */
+ * the first such read or write and kept.  Synchronises the stream.  After a
+ * step that gave up (OD_ETIMEOUT) dst is left as it was. */
 OD_API od_status od_read(od_ctx *ctx, double *dst, int32_t dst_is_device);
 
 /* Read n (0..2^24) cells of the current field into out (host), without
