@@ -382,12 +382,12 @@ constexpr int kIoRows = 4;
 // to export, and g stays as it is.
 __global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t ny, double *g, const FmtDev *fmt,
                          const ErrDev *err) {
-    const bool failed = err && err->code != 0;  // (looked at after the first cells are loaded)
+    const bool failed = err && err->code != 0;  // (needed with the first chare's extents, loaded beside them)
     const uint32_t base = fmt->base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (int c = blockIdx.y; c < nch; c += gridDim.y) {
         const ChareDev &C = ch[c];
-        const int nrow = C.by * C.bz, bx = C.bx;
+        const int nrow = failed ? 0 : C.by * C.bz, bx = C.bx;
         const int64_t plane = (int64_t)C.rows * C.pitch;
         for (int r0 = (blockIdx.x * nwarps + warp) * kIoRows; r0 < nrow; r0 += gridDim.x * nwarps * kIoRows) {
             const double *src[kIoRows];
@@ -403,7 +403,6 @@ __global__ void k_gather(const ChareDev *ch, int nch, int p, int64_t nx, int64_t
                 double v[kIoRows];
 #pragma unroll
                 for (int u = 0; u < kIoRows; ++u) v[u] = src[u][i];
-                if (failed) return;
 #pragma unroll
                 for (int u = 0; u < kIoRows; ++u)
                     dst[u][i] = fx_decode(f64_bits(v[u]), base);  // a repeated row stores the same value

@@ -151,12 +151,12 @@ static __device__ __noinline__ double update_slow(double W, double E, double S, 
 // given by its address in the planes below, of and above it.
 static __device__ __noinline__ double update_slow_fx(const double *sd, const double *sc, const double *su, int pitch,
                                                      uint32_t e0) {
-    double s = ieee_add(fx_decode(f64_bits(sc[-1]), e0), fx_decode(f64_bits(sc[1]), e0));
-    s = ieee_add(s, fx_decode(f64_bits(sc[-pitch]), e0));
-    s = ieee_add(s, fx_decode(f64_bits(sc[pitch]), e0));
-    s = ieee_add(s, fx_decode(f64_bits(*sd), e0));
-    s = ieee_add(s, fx_decode(f64_bits(*su), e0));
-    return f64_from(fx_encode(div6(s), e0));
+    double s = ieee_add(fx_decode_any(f64_bits(sc[-1]), e0), fx_decode_any(f64_bits(sc[1]), e0));
+    s = ieee_add(s, fx_decode_any(f64_bits(sc[-pitch]), e0));
+    s = ieee_add(s, fx_decode_any(f64_bits(sc[pitch]), e0));
+    s = ieee_add(s, fx_decode_any(f64_bits(*sd), e0));
+    s = ieee_add(s, fx_decode_any(f64_bits(*su), e0));
+    return f64_from(fx_encode_any(div6(s), e0));
 }
 
 // Which thread refills a ring slot: lane 0 of a different warp each plane
@@ -506,13 +506,13 @@ static __device__ __noinline__ double update2d_slow(double W, double E, double S
 
 static __device__ __noinline__ double update2d_slow_fx(const double *sd, const double *sc, const double *su,
                                                        uint32_t e0) {
-    double s = ieee_add(fx_decode(f64_bits(sc[-1]), e0), fx_decode(f64_bits(sc[1]), e0));
-    s = ieee_add(s, fx_decode(f64_bits(*sd), e0));
-    s = ieee_add(s, fx_decode(f64_bits(*su), e0));
+    double s = ieee_add(fx_decode_any(f64_bits(sc[-1]), e0), fx_decode_any(f64_bits(sc[1]), e0));
+    s = ieee_add(s, fx_decode_any(f64_bits(*sd), e0));
+    s = ieee_add(s, fx_decode_any(f64_bits(*su), e0));
     bool ok;
     double v = div4_fast(s, ok);
     if (!ok) v = ieee_div(s, 4.0);
-    return f64_from(fx_encode(v, e0));
+    return f64_from(fx_encode_any(v, e0));
 }
 
 // The 2D 5-point sweep (the paper's Jacobi2D, Sec. V) on the internal grid
